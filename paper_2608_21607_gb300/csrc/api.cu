@@ -654,7 +654,7 @@ nmd_status launch_update_rows(nmd_handle* h, const StepArgs& a, const Roles& ro,
   if (tc_update(h)) {
     const nmd_status st = launch_update_tc(sub, R + lo * h->rp, Rs + lo * h->rp, flags + lo, *gi_of(h, Ginv),
                                            (float)h->opt.eta, momentum ? (float)h->opt.gamma : 0.f, momentum,
-                                           h->ws.status, h->num_sms, s);
+                                           h->ws.status, s);
     if (st != NMD_OK) return fail(h, st, "tensor-core update");
   } else {
     launch_update(sub, R + lo * h->rp, Rs + lo * h->rp, flags + lo, Ginv, gsplit_of(h, Ginv), (float)h->opt.eta,

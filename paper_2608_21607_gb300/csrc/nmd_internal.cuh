@@ -304,8 +304,7 @@ nmd_status launch_embed(const Factor& W, const Factor& B, int64_t n, int r, int 
 // pieces each (gi: the pieces of G^{-1}, rp rows), the step applied to rows
 // [a.m0, a.m0 + a.M) of a.fm in its epilogue
 nmd_status launch_update_tc(const StepArgs& a, const float* R, const float* Rs, const uint8_t* flags,
-                            const Factor& gi, float eta, float gamma, bool momentum, int* status, int num_sms,
-                            cudaStream_t s);
+                            const Factor& gi, float eta, float gamma, bool momentum, int* status, cudaStream_t s);
 // Q-side rows per chunk of the tensor-core dense kernel (64 or 128)
 int panel_chunk_rows(int rp, int precision);
 // balls of the 128-row M tiles of rows [m0, m0 + M) of Xm and of the bn-row

@@ -23,14 +23,18 @@
 // summed by a separate pass.
 //
 // Warp roles (352 threads, one CTA per SM, persistent over M tiles):
-//   warps 0-7  epilogue, two warpgroups taking alternate chunks; in each,
-//              thread t owns TMEM lane t = tile row t
+//   warps 0-7  epilogue, two warpgroups; in each, thread t owns TMEM lane t =
+//              tile row t
 //   warp 8     TMA producer of Q chunks and W tiles (+ TMEM allocation)
 //   warp 9     issues MMA1 (L = W Q^T) for every chunk
 //   warp 10    issues MMA2 (R += P Q) for every chunk
-// The two MMA warps run converged and predicate each tcgen05 operation on an
-// elected lane; with two issuers the bookkeeping of one (barrier polls,
-// commits) overlaps the other's products on the tensor core.
+// The MMA warps run converged and predicate each tcgen05 operation on an
+// elected lane.
+// With two of them the bookkeeping of one (barrier tests, votes, branches: about
+// 200 cycles per chunk) runs while the other's MMAs keep the tensor core busy:
+// its queue holds next to nothing, a single issuer's bookkeeping is added to
+// every chunk (860 cycles per 128 x 128 chunk at r_pad = 64 against 512 of
+// products).
 // Every mbarrier wait is bounded (2 s): on expiry the kernel records
 // NMD_ERR_TIMEOUT, the other roles stop at their next wait, in-flight MMAs
 // and copies are drained and TMEM is freed before the kernel returns.
@@ -52,17 +56,23 @@ using namespace tc;
 constexpr int kEpiThreads = 256;                 // two epilogue warpgroups
 constexpr int kProducerWarp = 8, kMma1Warp = 9, kMma2Warp = 10;
 constexpr int kThreads = 352;
+// Launch bound of the panel kernel at r_pad <= 64: caps its registers at 128 a
+// thread, so that an update block (256 threads of 80) finds room in the
+// register file beside a CTA (352 x 128 + 256 x 80 = 65,536).
+constexpr int kRegThreads = 512;
 constexpr int BM = 128;
 constexpr uint64_t kTimeoutNs = 2000000000ull;
 
-template <int RP, bool SPLIT, bool LOSS>
+// SK: a chunk-skipping kernel (its chunk size is part of what
+// nmd_range_mask and nmd_skip_count report)
+template <int RP, bool SPLIT, bool LOSS, bool SK = false>
 struct Cfg {
   // fp32-accurate mode at r_pad = 256: W hi + lo take 256 TMEM columns, so a
   // CTA accumulates one 128-column half of R (blockIdx.y selects it) and the
   // first product is formed once per half
   static constexpr bool RHALF = SPLIT && !LOSS && RP == 256;
   static constexpr int NR = RHALF ? RP / 2 : RP;        // R columns of one CTA
-  // TMEM columns of the R accumulator; the loss pass has none.  In the bf16
+  // TMEM columns of one R accumulator; the loss pass has none.  In the bf16
   // mode the second product multiplies P by q_hi alone: the update pairs
   // this term with the Gram matrix of q_hi, so the rounding of q cancels
   // (see update_kernel), and R needs one accumulator of r_pad columns.
@@ -72,16 +82,25 @@ struct Cfg {
   // to the L buffers.
   static constexpr bool WSMEM = !SPLIT && !LOSS && RP <= 128;
   // Q rows per chunk (the N of the first product and the K of the second):
-  // 128 where three L buffers of 128 columns fit beside R (bf16 mode at
-  // r_pad <= 64: 3 x 128 + r_pad <= 512); 64 where that would leave fewer
-  // than three.  (Four buffers of 96 rows were slower at r_pad = 64.)
-  static constexpr int BN = WSMEM ? (RP == 128 ? 64 : 128) : ((RP == 256 || (SPLIT && RP == 128)) ? 64 : 128);
+  // 128 where at least two L buffers of 128 columns fit beside R and W, else
+  // 64.  A chunk of 64 rows reads the W tile from shared memory twice as
+  // often per product, which at r_pad = 128 takes longer than the product.
+  static constexpr int BN = WSMEM ? (RP == 128 && SK ? 64 : 128)
+                                  : ((RP == 256 || (SPLIT && RP == 128)) ? 64 : 128);
   // TMEM columns of one W tile (hi [+ lo]); none when it sits in shared memory
   static constexpr int WCOLS = WSMEM ? 0 : (SPLIT ? RP : RP / 2);
   static constexpr int W_BYTES = WSMEM ? BM * RP * 2 : 0;   // one W tile in shared memory
   static constexpr int NWB = (RP == 256) ? 1 : 2;      // W tile buffers
   static constexpr int FREE = 512 - NWB * WCOLS - RCOLS;
-  static constexpr int NB = FREE / BN >= 6 ? 6 : FREE / BN;  // L buffers
+  static constexpr int NB_MAX = LOSS ? 6 : (RP == 128 && !SPLIT && !SK ? 2 : 3);
+  static constexpr int NB = FREE / BN >= NB_MAX ? NB_MAX : FREE / BN;  // L buffers
+  // R accumulators: with two, the second product of the next tile starts
+  // while the epilogue still reads this tile's R
+  static constexpr int NRB = (!LOSS && NB * BN + 2 * RCOLS + NWB * WCOLS <= 512) ? 2 : 1;
+  // with two L buffers both epilogue warpgroups share every chunk (half of
+  // its columns each), which halves the time a buffer is held; with three
+  // they take alternate chunks (fewer hand-offs per element)
+  static constexpr bool HALF = !LOSS && NB == 2;
   static constexpr int PANEL_W = RP < 64 ? RP : 64;    // elements per row of one swizzle panel
   static constexpr int ROWB = PANEL_W * 2;             // bytes per panel row (= swizzle width)
   static constexpr int PANEL_BYTES = BN * ROWB;
@@ -91,26 +110,29 @@ struct Cfg {
   // and lo2 in the fp32-accurate mode (hi and lo in its loss pass)
   static constexpr int NQ = SPLIT ? (LOSS ? 2 : 3) : 1;
   static constexpr int STAGE_BYTES = OPER_BYTES * NQ;
-  // stages within 160 KB with the W tiles (r_pad <= 64: 165 KB in all, so
-  // that an update block fits beside the CTA), 192 KB at r_pad = 128
+  // R on its way out: 32 rows x 32 columns per epilogue warp
+  static constexpr int STG_BYTES = LOSS ? 0 : (kEpiThreads / 32) * 4096;
+  // stages within 160 KB with the W tiles and the R staging (r_pad <= 64: 165
+  // KB in all, so that an update block fits beside the CTA), 224 KB at r_pad =
+  // 128; beside the staging where W sits in TMEM
   static constexpr int NSTAGE_RAW =
-      ((WSMEM && RP <= 64) ? 160 * 1024 - NWB * W_BYTES : (WSMEM ? 192 * 1024 - NWB * W_BYTES : 160 * 1024)) /
-      STAGE_BYTES;
+      (WSMEM ? (RP <= 64 ? 160 : 224) * 1024 - NWB * W_BYTES - STG_BYTES : 160 * 1024) / STAGE_BYTES;
   static constexpr int NSTAGE = NSTAGE_RAW > 8 ? 8 : (NSTAGE_RAW < 2 ? 2 : NSTAGE_RAW);
   static constexpr uint32_t SWZ = PANEL_W == 64 ? SWZ_128B : (PANEL_W == 32 ? SWZ_64B : SWZ_32B);
-  // shared memory: stages, W tiles (WSMEM), barriers, TMEM slot + abort flag, ...
+  // shared memory: stages, W tiles (WSMEM), R staging, barriers, TMEM slot + abort flag, ...
   static constexpr size_t OFF_W = (size_t)NSTAGE * STAGE_BYTES;
   static constexpr int W_PANEL_BYTES = BM * ROWB;     // one swizzle panel of a W tile
-  static constexpr size_t OFF_BARS = OFF_W + (size_t)NWB * W_BYTES;
-  static constexpr int COL_L = 0;               // NB x BN columns
-  static constexpr int COL_R = NB * BN;         // RP columns
-  static constexpr int COL_W = COL_R + RCOLS;   // NWB x WCOLS columns
-  // barriers: full[NSTAGE], empty[NSTAGE], lfull[NB], pfull[NB], lfree[NB], rfull, rempty,
+  static constexpr size_t OFF_STG = OFF_W + (size_t)NWB * W_BYTES;
+  static constexpr size_t OFF_BARS = OFF_STG + STG_BYTES;
+  static constexpr int COL_L = 0;                     // NB x BN columns
+  static constexpr int COL_R = NB * BN;               // NRB x RCOLS columns
+  static constexpr int COL_W = COL_R + NRB * RCOLS;   // NWB x WCOLS columns
+  // barriers: full[NSTAGE], empty[NSTAGE], lfull[NB], pfull[NB], lfree[NB], rfull[2], rempty[2],
   // wfull[2], wempty[2], drain, drain2
-  static constexpr int NBAR = 2 * NSTAGE + 3 * NB + 8;
+  static constexpr int NBAR = 2 * NSTAGE + 3 * NB + 10;
   // after the barriers: TMEM slot and abort flag (64 B), the loss reduction
-  // (256 x 16 B), and 4 flags per L buffer (Delta form: P nonzero per warp)
-  static constexpr size_t SMEM_USED = 1024 + OFF_BARS + NBAR * 8 + 64 + 256 * 16 + NB * 16;
+  // (256 x 16 B), and 8 flags per L buffer (Delta form: P nonzero per warp)
+  static constexpr size_t SMEM_USED = 1024 + OFF_BARS + NBAR * 8 + 64 + (LOSS ? 256 * 16 : 0) + NB * 32;
   // at least 120 KB so that a second CTA (and its 512-column TMEM request)
   // never shares the SM
   static constexpr size_t SMEM = SMEM_USED > 120 * 1024 ? SMEM_USED : 120 * 1024;
@@ -118,6 +140,7 @@ struct Cfg {
   static_assert(NSTAGE >= 2, "stages");
   static_assert(SMEM <= 227 * 1024, "shared memory per block");
   static_assert(COL_W + NWB * WCOLS <= 512, "TMEM budget");
+  static_assert(LOSS || COL_R + (NRB - 1) * RCOLS + (RCOLS + 31) / 32 * 32 <= 512, "R is read 32 columns at a time");
   static_assert(BN % 32 == 0 && RP % 16 == 0, "shapes");
 };
 
@@ -190,25 +213,19 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile
   return wait_bar_slow(bar, parity, abort_flag, status, where);
 }
 
-// Wait for a converged warp: every lane tests the phase; if it has not
-// completed, lane 0 polls and the outcome is broadcast.
+// Wait of a converged warp, every lane testing the phase: `ready` is the
+// result of an earlier mbar_test_wait (a test takes about 60 cycles even when
+// the phase is complete, so the MMA warp starts it ahead of the instructions
+// it does not guard).
+__device__ __forceinline__ bool conv_wait(bool ready, uint32_t bar, uint32_t parity, volatile int* abort_flag,
+                                          int* status, int where) {
+  if (__all_sync(0xffffffffu, ready)) return true;
+  const bool ok = wait_bar_slow(bar, parity, abort_flag, status, where);
+  return __all_sync(0xffffffffu, ok);
+}
 __device__ __forceinline__ bool conv_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status,
                                           int where) {
-  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-  int ok = 0;
-  if ((threadIdx.x & 31) == 0) ok = wait_bar_slow(bar, parity, abort_flag, status, where);
-  ok = __shfl_sync(0xffffffffu, ok, 0);
-  return ok != 0;
-}
-
-// Warp-uniform wait: lane 0 polls, the outcome is broadcast to the warp.
-__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status,
-                                          int where) {
-  int ok = 0;
-  if ((threadIdx.x & 31) == 0) ok = wait_bar(bar, parity, abort_flag, status, where);
-  ok = __shfl_sync(0xffffffffu, ok, 0);
-  __syncwarp();
-  return ok != 0;
+  return conv_wait(mbar_try_wait(bar, parity), bar, parity, abort_flag, status, where);
 }
 
 // The live Q chunks [0, n) of one tile (this CTA's split of it starts at
@@ -263,6 +280,95 @@ __device__ __forceinline__ ChunkMask chunk_mask(const TcParams& p, int64_t t, in
   return cm;
 }
 
+// The live chunks of a CTA's tiles in order, as an MMA warp walks them: whether
+// the current chunk is its tile's first or last live one.  Without a
+// range-search mask this is a counter within the tile.
+template <bool RANGE>
+struct ChunkWalk {
+  int left, n, c, clast;   // tiles left (this one included), chunks per tile, current and last live chunk
+  bool first;
+  int t;                   // RANGE: the tile, its mask
+  int64_t kc0, nlive;
+  ChunkMask cm;
+  __device__ __forceinline__ ChunkWalk(const TcParams& p, int ntiles, int nchunks, int64_t kc0_)
+      : left((ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x), n(nchunks), t(blockIdx.x), kc0(kc0_) {
+    enter(p);
+  }
+  __device__ __forceinline__ void enter(const TcParams& p) {
+    c = 0;
+    first = true;
+    clast = n - 1;
+    if (!RANGE || left <= 0) return;
+    int64_t last;
+    cm = chunk_mask<RANGE>(p, t, kc0, n, &last, &nlive);
+    clast = (int)last;
+    while (!cm.live(c)) ++c;
+  }
+  __device__ __forceinline__ bool valid() const { return left > 0; }
+  __device__ __forceinline__ bool last() const { return c == clast; }
+  __device__ __forceinline__ void next(const TcParams& p) {
+    if (!RANGE) {   // (no branches: n >= 1)
+      first = c == clast;
+      left -= first ? 1 : 0;
+      c = first ? 0 : c + 1;
+      return;
+    }
+    if (last()) {
+      --left;
+      t += gridDim.x;
+      enter(p);
+      return;
+    }
+    first = false;
+    ++c;
+    while (!cm.live(c)) ++c;
+  }
+};
+
+// R of one 128-row tile from TMEM to global memory by one epilogue warp (rows
+// [li0, li0 + 32) of the step, lanes [lane_base ...) of TMEM): 32 columns at a
+// time through the warp's 4 KB of shared memory (16-byte pieces swizzled by
+// row), so that a store instruction covers whole 128-byte lines of four rows.
+// (Written straight from the TMEM layout, one row per lane, every 16-byte
+// store of a warp touched 32 lines: about 3,500 cycles per tile at r_pad = 64,
+// a tenth of the tile's time.)  Warpgroup wg takes every second group of 32
+// columns; the warp's last TMEM read releases the accumulator (b_rempty)
+// before the stores.  Called once per tile and warp, and kept out of line: the
+// hot loops of the epilogue and MMA warps then stay in the instruction caches.
+template <int NR, int RP>
+__device__ __noinline__ void store_r_tile(uint32_t tmem_r, uint32_t b_rempty, float* stg, float* dst, int64_t li0,
+                                          int64_t M, int wg, int lane) {
+  constexpr int NJ = (NR + 31) / 32;
+#pragma unroll 1
+  for (int j = wg; j < NJ; j += 2) {
+    uint32_t v[32];
+    tmem_ld32(tmem_r + j * 32, v);   // RP = 16 reads 16 columns past R
+    tmem_wait_ld(v);
+    if (j + 2 >= NJ) {
+      fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(b_rempty);
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      *(uint4*)(stg + lane * 32 + ((k ^ (lane & 7)) << 2)) = make_uint4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+    __syncwarp();
+    const int ch = lane & 7;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int rr = 4 * u + (lane >> 3);
+      if (li0 + rr < M && j * 32 + 4 * ch < NR)
+        *(float4*)(dst + (int64_t)rr * RP + j * 32 + 4 * ch) = *(const float4*)(stg + rr * 32 + ((ch ^ (rr & 7)) << 2));
+    }
+    __syncwarp();   // the buffer is refilled by the next 32 columns
+  }
+  if (wg >= NJ) {   // no columns for this warpgroup (r_pad <= 32): release at once
+    fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(b_rempty);
+  }
+}
+
 // MODE: 0 the panel contraction R = P(L) Q; 1 the loss pass (first product
 // only, sums of max(0, L)^2 and max(0, L) off the support); 2 the nearest-
 // neighbour pass (first product only, per row the largest L_ij, j != i);
@@ -273,7 +379,7 @@ __device__ __forceinline__ ChunkMask chunk_mask(const TcParams& p, int64_t t, in
 // products of the chunks that the range-search mask clears.  Separate
 // instantiations, so that the kernel without them carries none of the checks.
 template <int RP, int EPI, bool SPLIT, int MODE, int SKIPM>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(MODE == 0 ? kRegThreads : kThreads, 1)
     panel_tc_kernel(const __grid_constant__ CUtensorMap tq_hi, const __grid_constant__ CUtensorMap tq_lo,
                     const __grid_constant__ CUtensorMap tq_lo2, const __grid_constant__ CUtensorMap tw,
                     const TcParams p) {
@@ -283,9 +389,18 @@ __global__ void __launch_bounds__(kThreads, 1)
   // the update is skipped under a sticky error (as the CUDA-core update is);
   // every thread reads the same word before any barrier or TMEM exists
   if (UPDATE && *(volatile int*)p.status != 0) return;
-  using C = Cfg<RP, SPLIT, LOSS>;
+  using C = Cfg<RP, SPLIT, LOSS, SKIPM != 0>;
   constexpr int BN = C::BN, NB = C::NB, NSTAGE = C::NSTAGE, NWB = C::NWB;
   constexpr bool VOTE = SKIPM == 1, RANGE = SKIPM == 2;
+  // One warp issues both products (see the MMA1 issuer) where a chunk's MMAs
+  // take longer than a warp's bookkeeping: 103 -> 93 us at r_pad = 64 and 167 ->
+  // 158 us at r_pad = 128 (bf16; 139,255 rows against 4,096), 537 -> 527 us at
+  // r_pad = 128 in the fp32-accurate mode.  At r_pad <= 32 two warps share the
+  // bookkeeping (65 against 81 us at r_pad = 16), and so they do in the
+  // fp32-accurate mode at r_pad = 64 (281 against 290 us), with one W buffer or
+  // as many stages as L buffers (r_pad = 256: MMA1 must not hold up MMA2 while
+  // it waits for them), and with a range-search mask.
+  constexpr bool ONE_MMA = !LOSS && !RANGE && NWB == 2 && NSTAGE > NB && (RP == 128 || (RP == 64 && !SPLIT));
   static_assert(SKIPM == 0 || (EPI == 1 && !LOSS), "skipping is a Delta-form option");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -295,7 +410,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t* tmem_slot = (uint32_t*)(bars + C::NBAR);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
   double* red = (double*)(smem + C::OFF_BARS + C::NBAR * 8 + 64);
-  volatile uint32_t* pflag = (volatile uint32_t*)(red + 2 * kEpiThreads);   // [NB][4]
+  volatile uint32_t* pflag = (volatile uint32_t*)red;   // [NB][8] (panel kernel; it has no reduction)
 
   const uint32_t b_full = smem_u32(bars);
   const uint32_t b_empty = b_full + 8 * NSTAGE;
@@ -303,13 +418,15 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t b_pfull = b_lfull + 8 * NB;
   const uint32_t b_lfree = b_pfull + 8 * NB;
   const uint32_t b_rfull = b_lfree + 8 * NB;
-  const uint32_t b_rempty = b_rfull + 8;
-  const uint32_t b_wfull = b_rempty + 8;
+  const uint32_t b_rempty = b_rfull + 16;
+  const uint32_t b_wfull = b_rempty + 16;
   const uint32_t b_wempty = b_wfull + 16;
   const uint32_t b_drain = b_wempty + 16;
   const uint32_t b_drain2 = b_drain + 8;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // (broadcast, so that the compiler knows the roles' branches are uniform and
+  // keeps the MMA warp's addresses and descriptors in uniform registers)
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int i = 0; i < NSTAGE; ++i) {
       mbar_init(b_full + 8 * i, 1);
@@ -317,12 +434,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int i = 0; i < NB; ++i) {
       mbar_init(b_lfull + 8 * i, 1);
-      mbar_init(b_pfull + 8 * i, 4);                 // the four warps of one epilogue warpgroup
-      mbar_init(b_lfree + 8 * i, LOSS ? 4 : 1);
+      mbar_init(b_pfull + 8 * i, C::HALF ? 8 : 4);   // the warps of both epilogue warpgroups, or of one
+      mbar_init(b_lfree + 8 * i, LOSS ? 4 : 1);      // one warpgroup, or MMA2's commit
     }
-    mbar_init(b_rfull, 1);
-    mbar_init(b_rempty, kEpiThreads / 32);
     for (int i = 0; i < 2; ++i) {
+      mbar_init(b_rfull + 8 * i, 1);
+      mbar_init(b_rempty + 8 * i, kEpiThreads / 32);
       mbar_init(b_wfull + 8 * i, C::WSMEM ? 1 : kEpiThreads / 32);   // TMA, or the epilogue warps
       mbar_init(b_wempty + 8 * i, 1);
     }
@@ -353,6 +470,69 @@ __global__ void __launch_bounds__(kThreads, 1)
   float* const Rout = p.ksplit ? p.R + kz * p.rstride : p.R;
   const int64_t nchunks = (kK + BN - 1) / BN;
   const int64_t kc0 = (kq0 - p.q0) / BN;   // this CTA's first chunk within the tile's mask
+
+  // The MMAs of one chunk's products (issued by a converged warp).  Descriptors:
+  // only the start address varies; WSMEM: the W tile in the same K-major
+  // swizzled panels as a chunk.
+  // In the Z form of the bf16 mode MMA1 forms -L (its A operand negated), so
+  // that the epilogue needs one conversion with a clamp at zero, P = max(0,
+  // -L), and MMA2 negates it: -P = min(0, L).
+  constexpr bool NEG1 = MODE == 0 && EPI == 0 && !SPLIT;
+  const uint64_t dq1 = sdesc(smem_u32(stages), 16, 8 * C::ROWB, C::SWZ);   // a chunk, K-major
+  const uint64_t dw = sdesc(wsm0, 16, 8 * C::ROWB, C::SWZ);
+  auto mma1 = [&](int st, int lb, int wb) {
+    constexpr uint32_t idesc1 = idesc_bf16(BM, BN, false, NEG1);
+    const uint32_t wh = tmem + C::COL_W + wb * C::WCOLS, wl = wh + RP / 2;
+    const uint32_t bo = (uint32_t)st * (C::STAGE_BYTES >> 4), ao = (uint32_t)wb * (C::W_BYTES >> 4);
+    const uint32_t d = tmem + C::COL_L + lb * BN;
+#pragma unroll
+    for (int k = 0; k < RP / 16; ++k) {
+      constexpr int PW = C::PANEL_W;
+      const uint32_t off = bo + (((k * 16 / PW) * C::PANEL_BYTES + ((k * 16) % PW) * 2) >> 4);
+      const uint32_t aoff = ao + (((k * 16 / PW) * C::W_PANEL_BYTES + ((k * 16) % PW) * 2) >> 4);
+      if (C::WSMEM) mma_ss_elect(d, dw, aoff, dq1, off, idesc1, k > 0);
+      else mma_ts_elect(d, wh + k * 8, dq1, off, idesc1, k > 0);
+      if (SPLIT) {
+        mma_ts_elect(d, wh + k * 8, dq1, off + (C::OPER_BYTES >> 4), idesc1, 1);
+        mma_ts_elect(d, wl + k * 8, dq1, off, idesc1, 1);
+      }
+    }
+  };
+  // R columns [hcol, hcol + NR) of Q: their panels start hcol / PANEL_W panels in
+  const uint32_t hpan = C::RHALF ? (uint32_t)blockIdx.y * (C::NR / C::PANEL_W) * C::PANEL_BYTES : 0u;
+  const uint64_t dq2 = sdesc(smem_u32(stages) + hpan, C::PANEL_BYTES, 8 * C::ROWB, C::SWZ);   // a chunk, MN-major
+  auto mma2 = [&](int st, int lb, int rb, bool accumulate) {
+    constexpr uint32_t idesc2 = idesc_bf16(BM, LOSS ? 16 : C::NR, true, !SPLIT);
+    const uint32_t bo = (uint32_t)st * (C::STAGE_BYTES >> 4);
+    const uint32_t pl = tmem + C::COL_L + lb * BN;
+    const uint32_t dr = tmem + C::COL_R + rb * C::RCOLS;
+#pragma unroll
+    for (int k = 0; k < BN / 16; ++k) {
+      const uint32_t off = bo + ((k * 16 * C::ROWB) >> 4);
+      const uint32_t acc = k > 0 || accumulate ? 1u : 0u;
+      if (!SPLIT) {             // P q_hi; each warpgroup's P starts at its own columns of L
+        constexpr int KH = BN / 32;   // k steps per half
+        mma_ts_elect(dr, pl + (C::HALF ? (k / KH) * (BN / 2) + (k % KH) * 8 : k * 8), dq2, off, idesc2, acc);
+      } else {                  // P_hi (q_hi + q_lo + q_lo2) + P_lo q_hi
+        const uint32_t ph = pl + (k / 2) * 32 + (k % 2) * 8, plo = ph + 16;
+        mma_ts_elect(dr, ph, dq2, off, idesc2, acc);
+        mma_ts_elect(dr, ph, dq2, off + (C::OPER_BYTES >> 4), idesc2, 1);
+        mma_ts_elect(dr, ph, dq2, off + ((2 * C::OPER_BYTES) >> 4), idesc2, 1);
+        mma_ts_elect(dr, plo, dq2, off, idesc2, 1);
+      }
+    }
+  };
+  // Delta form: a chunk whose P is zero in every row adds nothing to R (Sec.
+  // 4.3); its MMAs are skipped, except for the first chunk of a tile, which
+  // initialises the accumulator
+  auto vanishes = [&](int lb, bool first) -> bool {
+    if (!VOTE || first) return false;
+    uint32_t nz = 0u;
+#pragma unroll
+    for (int w = 0; w < (C::HALF ? 8 : 4); ++w) nz |= pflag[8 * lb + w];
+    if (nz == 0u && p.skips != nullptr && lane == 0) atomicAdd(p.skips, 1ull);
+    return nz == 0u;
+  };
 
   if (warp == kProducerWarp) {
     // ------------------------------------------------------------ producer
@@ -411,53 +591,92 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == kMma1Warp) {
     // ------------------------------------------------------------ MMA1 issuer
-    // L[lb] = W tile x chunk^T for every chunk G of this CTA's tiles, in order.
-    constexpr uint32_t idesc1 = idesc_bf16(BM, BN, false);   // Q K-major
-    const uint32_t stage0 = smem_u32(stages);
+    // L[lb] = W tile x chunk^T for every chunk of this CTA's tiles, in order;
+    // with ONE_MMA also R += P[lb] x chunk.
     int s1 = 0, l1 = 0, wb1 = 0;
     uint32_t ph_full = 0, ph_lfree = 1, ph_wfull = 0;
-    bool ok = true;
-    for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-      int64_t clast, nlive;
-      const ChunkMask cm = chunk_mask<RANGE>(p, t, kc0, nchunks, &clast, &nlive);
-      if (RANGE && p.skips != nullptr && lane == 0 && nlive < nchunks)
-        atomicAdd(p.skips, (unsigned long long)(nchunks - nlive));
-      bool first = true;
-      for (int64_t c = 0; c < nchunks; ++c) {
-        if (RANGE && !cm.live(c)) continue;
-        if (first && !(ok = conv_wait(b_wfull + 8 * wb1, ph_wfull, abort_flag, p.status, 2))) break;
-        first = false;
-        if (!(ok = conv_wait(b_full + 8 * s1, ph_full, abort_flag, p.status, 3))) break;
-        if (!(ok = conv_wait(b_lfree + 8 * l1, ph_lfree, abort_flag, p.status, 4))) break;
+    ChunkWalk<RANGE> k1(p, (int)ntiles, (int)nchunks, kc0);
+    auto advance1 = [&](bool last) {
+      s1 = s1 == NSTAGE - 1 ? 0 : s1 + 1;
+      ph_full ^= s1 == 0 ? 1u : 0u;
+      l1 = l1 == NB - 1 ? 0 : l1 + 1;
+      ph_lfree ^= l1 == 0 ? 1u : 0u;
+      if (NWB == 2) wb1 ^= last ? 1 : 0;
+      ph_wfull ^= (last && wb1 == 0) ? 1u : 0u;
+      k1.next(p);
+    };
+    if constexpr (ONE_MMA) {
+      // MMA1 runs NB chunks ahead of MMA2, and MMA1 of chunk c + NB goes right
+      // behind MMA2 of chunk c: one thread's MMAs execute in issue order, so
+      // the L buffer that MMA2(c) reads can be overwritten by the next MMA in
+      // the queue, without waiting for MMA2's completion.  The queue holds
+      // next to nothing, so what stands between two batches of MMAs adds to
+      // the chunk: each barrier test (about 60 cycles) starts one batch
+      // before its result is needed, and the state advances without branches.
+      int s2 = 0, l2 = 0, rb2 = 0;
+      uint32_t ph_pfull = 0, ph_rempty = 1;
+      ChunkWalk<RANGE> k2 = k1;
+      bool ok = true;
+      for (int i = 0; i < NB && k1.valid() && ok; ++i) {
+        ok = conv_wait(b_full + 8 * s1, ph_full, abort_flag, p.status, 3) &&
+             (!k1.first || conv_wait(b_wfull + 8 * wb1, ph_wfull, abort_flag, p.status, 2));
+        if (!ok) break;
         fence_after();
-        const uint32_t wh = tmem + C::COL_W + wb1 * C::WCOLS;
-        const uint32_t wl = wh + RP / 2;
-        const uint64_t d1 = sdesc(stage0 + s1 * C::STAGE_BYTES, 16, 8 * C::ROWB, C::SWZ);
-        // WSMEM: the W tile in the same K-major swizzled panels as a chunk
-        const uint64_t a1 = sdesc(wsm0 + wb1 * C::W_BYTES, 16, 8 * C::ROWB, C::SWZ);
-        const uint32_t d = tmem + C::COL_L + l1 * BN;
-#pragma unroll
-        for (int k = 0; k < RP / 16; ++k) {
-          const uint32_t off = (k * 16 / C::PANEL_W) * C::PANEL_BYTES + ((k * 16) % C::PANEL_W) * 2;
-          const uint64_t bh = d1 + (off >> 4);
-          if (C::WSMEM)
-            mma_ss_elect(d, a1 + (((k * 16 / C::PANEL_W) * C::W_PANEL_BYTES + ((k * 16) % C::PANEL_W) * 2) >> 4), bh,
-                         idesc1, k > 0);
-          else
-            mma_ts_elect(d, wh + k * 8, bh, idesc1, k > 0);
-          if (SPLIT) {
-            const uint64_t bl = d1 + ((C::OPER_BYTES + off) >> 4);
-            mma_ts_elect(d, wh + k * 8, bl, idesc1, 1);
-            mma_ts_elect(d, wl + k * 8, bh, idesc1, 1);
-          }
+        const bool last = k1.last();
+        mma1(s1, l1, wb1);
+        commit_elect(b_lfull + 8 * l1);
+        if (last) commit_elect(b_wempty + 8 * wb1);
+        advance1(last);
+      }
+      bool pready = false;
+      while (ok && k2.valid()) {
+        if (!pready && !conv_wait(b_pfull + 8 * l2, ph_pfull, abort_flag, p.status, 5)) break;
+        if (k2.first && !conv_wait(b_rempty + 8 * rb2, ph_rempty, abort_flag, p.status, 6)) break;
+        fence_after();
+        const bool fr = mbar_test_wait(b_full + 8 * s1, ph_full);
+        const bool last2 = k2.last();
+        if (!vanishes(l2, k2.first)) mma2(s2, l2, rb2, !k2.first);
+        commit_elect(b_empty + 8 * s2);
+        if (last2) commit_elect(b_rfull + 8 * rb2);
+        s2 = s2 == NSTAGE - 1 ? 0 : s2 + 1;
+        l2 = l2 == NB - 1 ? 0 : l2 + 1;
+        ph_pfull ^= l2 == 0 ? 1u : 0u;
+        if (C::NRB == 2) rb2 ^= last2 ? 1 : 0;
+        ph_rempty ^= (last2 && rb2 == 0) ? 1u : 0u;
+        k2.next(p);
+        const bool pr = mbar_test_wait(b_pfull + 8 * l2, ph_pfull);
+        if (k1.valid()) {
+          if (!__all_sync(0xffffffffu, fr) && !conv_wait(b_full + 8 * s1, ph_full, abort_flag, p.status, 3)) break;
+          if (k1.first && !conv_wait(b_wfull + 8 * wb1, ph_wfull, abort_flag, p.status, 2)) break;
+          fence_after();
+          const bool last1 = k1.last();
+          mma1(s1, l1, wb1);
+          commit_elect(b_lfull + 8 * l1);
+          if (last1) commit_elect(b_wempty + 8 * wb1);
+          advance1(last1);
         }
+        pready = __all_sync(0xffffffffu, pr);
+      }
+    } else {
+      while (k1.valid()) {
+        const bool ready = mbar_test_wait(b_full + 8 * s1, ph_full) & mbar_test_wait(b_lfree + 8 * l1, ph_lfree);
+        if (!__all_sync(0xffffffffu, ready) &&
+            (!conv_wait(b_full + 8 * s1, ph_full, abort_flag, p.status, 3) ||
+             !conv_wait(b_lfree + 8 * l1, ph_lfree, abort_flag, p.status, 4)))
+          break;
+        if (k1.first) {
+          if (!conv_wait(b_wfull + 8 * wb1, ph_wfull, abort_flag, p.status, 2)) break;
+          if (RANGE && p.skips != nullptr && lane == 0 && k1.nlive < k1.n)
+            atomicAdd(p.skips, (unsigned long long)(k1.n - k1.nlive));
+        }
+        fence_after();
+        const bool last = k1.last();
+        mma1(s1, l1, wb1);
         commit_elect(b_lfull + 8 * l1);
         if (LOSS) commit_elect(b_empty + 8 * s1);
-        if (c == clast) commit_elect(b_wempty + 8 * wb1);
-        if (++s1 == NSTAGE) { s1 = 0; ph_full ^= 1u; }
-        if (++l1 == NB) { l1 = 0; ph_lfree ^= 1u; }
+        if (last) commit_elect(b_wempty + 8 * wb1);
+        advance1(last);
       }
-      if (++wb1 == NWB) { wb1 = 0; ph_wfull ^= 1u; }
     }
     // wait until every MMA issued by this warp has completed
     commit_elect(b_drain);
@@ -471,56 +690,26 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ------------------------------------------------------------ MMA2 issuer
     // R += P[lb] x chunk for every chunk once its P is in TMEM; frees the
     // shared-memory stage and the L buffer, and hands R over per tile.
-    if (!LOSS) {
-      constexpr uint32_t idesc2 = idesc_bf16(BM, C::NR, true, EPI == 1 && !SPLIT);   // Q MN-major
-      // R columns [hcol, hcol + NR) of Q: their panels start hcol / PANEL_W panels in
-      const uint32_t hpan = C::RHALF ? (uint32_t)blockIdx.y * (C::NR / C::PANEL_W) * C::PANEL_BYTES : 0u;
-      const uint32_t stage0 = smem_u32(stages);
-      int s2 = 0, l2 = 0;
+    if constexpr (!LOSS && !ONE_MMA) {
+      int s2 = 0, l2 = 0, rb2 = 0;
       uint32_t ph_pfull = 0, ph_rempty = 1;
-      bool ok = true;
-      for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-        int64_t clast, nlive;
-        const ChunkMask cm = chunk_mask<RANGE>(p, t, kc0, nchunks, &clast, &nlive);
-        bool first = true;
-        for (int64_t c = 0; c < nchunks; ++c) {
-          if (RANGE && !cm.live(c)) continue;
-          if (!(ok = conv_wait(b_pfull + 8 * l2, ph_pfull, abort_flag, p.status, 5))) break;
-          if (first && !(ok = conv_wait(b_rempty, ph_rempty, abort_flag, p.status, 6))) break;
-          fence_after();
-          // Delta form: a chunk whose P is zero in every row adds nothing to R
-          // (Sec. 4.3); its MMAs are skipped, except for the first chunk of a
-          // tile, which initialises the accumulator
-          bool skip = false;
-          if (VOTE && !first)
-            skip = (pflag[4 * l2] | pflag[4 * l2 + 1] | pflag[4 * l2 + 2] | pflag[4 * l2 + 3]) == 0u;
-          if (VOTE && skip && p.skips != nullptr && lane == 0) atomicAdd(p.skips, 1ull);
-          const uint64_t d2 = sdesc(stage0 + s2 * C::STAGE_BYTES + hpan, C::PANEL_BYTES, 8 * C::ROWB, C::SWZ);
-          const uint32_t pl = tmem + C::COL_L + l2 * BN;
-#pragma unroll
-          for (int k = 0; k < BN / 16 && !(VOTE && skip); ++k) {
-            const uint64_t bh = d2 + ((k * 16 * C::ROWB) >> 4);
-            const uint32_t acc = (!first || k > 0) ? 1u : 0u;
-            if (!SPLIT) {             // P q_hi
-              mma_ts_elect(tmem + C::COL_R, pl + k * 8, bh, idesc2, acc);
-            } else {                  // P_hi (q_hi + q_lo + q_lo2) + P_lo q_hi
-              const uint64_t bl = bh + (C::OPER_BYTES >> 4);
-              const uint64_t bl2 = bh + ((2 * C::OPER_BYTES) >> 4);
-              const uint32_t ph = pl + (k / 2) * 32 + (k % 2) * 8, plo = ph + 16;
-              mma_ts_elect(tmem + C::COL_R, ph, bh, idesc2, acc);
-              mma_ts_elect(tmem + C::COL_R, ph, bl, idesc2, 1);
-              mma_ts_elect(tmem + C::COL_R, ph, bl2, idesc2, 1);
-              mma_ts_elect(tmem + C::COL_R, plo, bh, idesc2, 1);
-            }
-          }
-          commit_elect(b_empty + 8 * s2);
-          commit_elect(b_lfree + 8 * l2);
-          if (c == clast) commit_elect(b_rfull);
-          if (++s2 == NSTAGE) s2 = 0;
-          if (++l2 == NB) { l2 = 0; ph_pfull ^= 1u; }
-          if (first) ph_rempty ^= 1u;
-          first = false;
-        }
+      ChunkWalk<RANGE> k2(p, (int)ntiles, (int)nchunks, kc0);
+      while (k2.valid()) {
+        if (!conv_wait(mbar_test_wait(b_pfull + 8 * l2, ph_pfull), b_pfull + 8 * l2, ph_pfull, abort_flag, p.status, 5))
+          break;
+        if (k2.first && !conv_wait(b_rempty + 8 * rb2, ph_rempty, abort_flag, p.status, 6)) break;
+        fence_after();
+        const bool last = k2.last();
+        if (!vanishes(l2, k2.first)) mma2(s2, l2, rb2, !k2.first);
+        commit_elect(b_lfree + 8 * l2);
+        commit_elect(b_empty + 8 * s2);
+        if (last) commit_elect(b_rfull + 8 * rb2);
+        s2 = s2 == NSTAGE - 1 ? 0 : s2 + 1;
+        l2 = l2 == NB - 1 ? 0 : l2 + 1;
+        ph_pfull ^= l2 == 0 ? 1u : 0u;
+        if (C::NRB == 2) rb2 ^= last ? 1 : 0;
+        ph_rempty ^= (last && rb2 == 0) ? 1u : 0u;
+        k2.next(p);
       }
       commit_elect(b_drain2);
       if (lane == 0) {
@@ -532,9 +721,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else {
     // ------------------------------------------------------------ epilogue
-    // Two warpgroups take alternate chunks; within a warpgroup thread t owns
-    // TMEM lane t = tile row t.  Tile-level work (W load, R readout) is split
-    // by columns between the two warpgroups.
+    // Two warpgroups take alternate chunks (HALF: half of every chunk's
+    // columns each); within a warpgroup thread t owns TMEM lane t = tile row
+    // t.  Tile-level work (W load, R readout) is split by columns between the
+    // two warpgroups.
     const int wg = warp >> 2;
     const int row = (warp & 3) * 32 + lane;
     const int et = threadIdx.x;                          // 0 .. 255
@@ -609,58 +799,159 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (lane == 0) mbar_arrive(b_wfull + 8 * wb);
     };
 
+    // Loss pass: this row's entries in columns [c0, c0 + BN) as bits, the row's
+    // position moved past them.  A row's first entries of the chunk are read
+    // by its own thread; what is left of a longer one (a hub of the graph has
+    // an entry in every column, 128 dependent loads per chunk) by the whole warp,
+    // 32 entries at a time.  The other warpgroup's chunks are passed over by
+    // a doubling search.  Called by converged warps.
+    auto support_mask = [&](int64_t c0, uint32_t(&msk)[BN / 32]) {
+      constexpr int W = BN / 32, kOwn = 8;
+      const int64_t cend = c0 + BN;
+#pragma unroll
+      for (int w = 0; w < W; ++w) msk[w] = 0u;
+      if (snext < c0) {   // first entry at or past column c0
+        int64_t step = 1, lo = se;   // cidx[lo] < c0
+        while (lo + step < send && p.cidx[lo + step] < c0) {
+          lo += step;
+          step *= 2;
+        }
+        int64_t hi = lo + step < send ? lo + step : send;
+        while (hi - lo > 1) {
+          const int64_t mid = lo + (hi - lo) / 2;
+          if (p.cidx[mid] < c0) lo = mid;
+          else hi = mid;
+        }
+        se = hi;
+        snext = se < send ? p.cidx[se] : INT64_MAX;
+      }
+      for (int n = 0; n < kOwn && snext < cend; ++n) {
+        const int b = (int)(snext - c0);
+#pragma unroll
+        for (int w = 0; w < W; ++w)
+          if (w == (b >> 5)) msk[w] |= 1u << (b & 31);
+        ++se;
+        snext = se < send ? p.cidx[se] : INT64_MAX;
+      }
+      uint32_t more = __ballot_sync(0xffffffffu, snext < cend);
+      while (more) {
+        const int src = __ffs(more) - 1;
+        more &= more - 1;
+        int64_t q = __shfl_sync(0xffffffffu, se, src);
+        const int64_t e = __shfl_sync(0xffffffffu, send, src);
+        uint32_t m[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) m[w] = 0u;
+        int n;
+        do {
+          const int64_t col = q + lane < e ? (int64_t)p.cidx[q + lane] : INT64_MAX;
+          const bool in = col < cend;
+          const int b = in ? (int)(col - c0) : 0;
+#pragma unroll
+          for (int w = 0; w < W; ++w)
+            m[w] |= __reduce_or_sync(0xffffffffu, in && (b >> 5) == w ? 1u << (b & 31) : 0u);
+          n = __popc(__ballot_sync(0xffffffffu, in));
+          q += n;
+        } while (n == 32);
+        if (lane == src) {
+#pragma unroll
+          for (int w = 0; w < W; ++w) msk[w] |= m[w];
+          se = q;
+          snext = se < send ? p.cidx[se] : INT64_MAX;
+        }
+      }
+    };
+
+    // R of a tile, the n-th of this CTA
+    auto readout = [&](int tile, int n) -> bool {
+      const int rb = n % C::NRB;
+      if (!conv_wait(b_rfull + 8 * rb, (uint32_t)((n / C::NRB) & 1), abort_flag, p.status, 8)) return false;
+      fence_after();
+      const int64_t li0 = (int64_t)tile * BM + (warp & 3) * 32;
+      if constexpr (MODE == 0)
+        store_r_tile<C::NR, RP>(tmem + lane_base + C::COL_R + rb * C::RCOLS, b_rempty + 8 * rb,
+                                (float*)(smem + C::OFF_STG) + warp * 1024,
+                                Rout + li0 * RP + (C::RHALF ? (int64_t)blockIdx.y * C::NR : 0), li0, p.M, wg, lane);
+      return true;
+    };
+
     {  // prologue: the first NWB tiles
-      int64_t tt = 0;
-      for (int64_t t = blockIdx.x; t < ntiles && tt < NWB; t += gridDim.x, ++tt) load_w(t, (int)tt);
+      int tt = 0;
+      for (int t = blockIdx.x; t < (int)ntiles && tt < NWB; t += gridDim.x, ++tt) load_w(t, tt);
     }
-    int64_t tt = 0;
-    int64_t Gc = 0;   // chunks this CTA has processed
-    for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tt) {
+    int tt = 0;          // tiles this CTA has processed
+    int lb = NB - 1;     // L buffer of the current chunk and the parity of its use
+    uint32_t lpar = 1;
+    bool odd = true;     // the chunks alternate between the warpgroups
+    int pend = -1;       // a tile whose R is still to be read out (NRB = 2)
+    for (int t = blockIdx.x; t < (int)ntiles && ok; t += gridDim.x, ++tt) {
       int64_t clast, nlive;
       const ChunkMask cm = chunk_mask<RANGE>(p, t, kc0, nchunks, &clast, &nlive);
       if (SUMS) {
-        const int64_t li = t * BM + row;
+        const int64_t li = (int64_t)t * BM + row;
         se = li < p.M ? p.rowptr[li] : 0;
         send = li < p.M ? p.rowptr[li + 1] : 0;
         snext = se < send ? p.cidx[se] : INT64_MAX;
       }
-      for (int64_t c = 0; c < nchunks; ++c) {
-        if (RANGE && !cm.live(c)) continue;
-        const int64_t G = Gc++;
-        if ((int)(G & 1) != wg) continue;
-        if (SUMS) {   // skip the support columns of the other warpgroup's chunks
-          while (snext < c * BN) {
-            ++se;
-            snext = se < send ? p.cidx[se] : INT64_MAX;
-          }
-        }
-        const int lb = (int)(G % NB);
-        if (!(ok = warp_wait(b_lfull + 8 * lb, (uint32_t)((G / NB) & 1), abort_flag, p.status, 7))) break;
+      for (int ci = 0; ci < (int)nchunks; ++ci) {
+        if (RANGE && !cm.live(ci)) continue;
+        const int64_t c = ci;
+        if (++lb == NB) { lb = 0; lpar ^= 1u; }
+        odd = !odd;
+        if (!C::HALF && odd != (wg != 0)) continue;
+        // the support columns of this chunk, one bit each, found while the
+        // chunk's product is under way: bit i of msk[g] = column 32 g + i
+        uint32_t msk[BN / 32];
+        if (SUMS) support_mask(c * BN, msk);
+        if (!(ok = conv_wait(b_lfull + 8 * lb, lpar, abort_flag, p.status, 7))) break;
         fence_after();
         const int kv = (int)(kK - c * BN < BN ? kK - c * BN : BN);   // valid columns in this chunk
         const uint32_t lcol = tmem + lane_base + C::COL_L + lb * BN;
         float c2 = 0.f, c1 = 0.f;
         uint32_t nzacc = 0u;   // Delta form: OR of this thread's P words
-        // one group of 32 columns of L (TMEM columns [32 g, 32 g + 32) of the
-        // buffer): mask the columns past the block, then the loss sums or P
-        // (bf16, 16 TMEM columns at 16 g; fp32-accurate: hi and lo, 32 at 32 g,
-        // so P never overwrites L columns that are still to be read)
+        // MODE 0: P of one group of 32 columns of L (TMEM columns [32 g, 32 g + 32)
+        // of the buffer): bf16, 16 TMEM columns at 16 g (HALF: within the
+        // warpgroup's own half of the buffer); fp32-accurate: hi and lo, 32 at 32
+        // g.  P never overwrites L columns that are still to be read.
+        auto to_p = [&](const uint32_t(&v)[32], int g) {
+          if (!SPLIT) {
+            // max(0, L) (Delta form) or max(0, -L) (Z form, v holds -L); MMA2
+            // negates both.  A NaN stays a NaN.
+            uint32_t pk[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              pk[i] = pack_relu_bf16x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+              if (VOTE) nzacc |= pk[i] & 0x7fff7fffu;   // -0 counts as zero
+            }
+            tmem_st16(C::HALF ? lcol + wg * (BN / 2) + (g - wg * (BN / 64)) * 16 : lcol + g * 16, pk);
+          } else {
+            // fp32-accurate: P = hi + lo, hi at columns [32 g, 32 g + 16), lo at [32 g + 16, 32 g + 32)
+            uint32_t ph[16], pl[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const float x0 = __uint_as_float(v[2 * i]), x1 = __uint_as_float(v[2 * i + 1]);
+              const float e0 = EPI == 0 ? fminf(0.f, x0) : fminf(0.f, -x0);
+              const float e1 = EPI == 0 ? fminf(0.f, x1) : fminf(0.f, -x1);
+              const uint32_t hp = pack_bf16x2(e0, e1);
+              const float h0 = __uint_as_float(hp << 16), h1 = __uint_as_float(hp & 0xffff0000u);
+              ph[i] = hp;
+              pl[i] = pack_bf16x2(e0 - h0, e1 - h1);
+              if (VOTE) nzacc |= (ph[i] | pl[i]) & 0x7fff7fffu;   // -0 counts as zero
+            }
+            tmem_st16(lcol + g * 32, ph);
+            tmem_st16(lcol + g * 32 + 16, pl);
+          }
+        };
+        // the first-product passes: one group of 32 columns, columns past the
+        // Q side masked
         auto group = [&](uint32_t(&v)[32], int g) {
-          if (kv < BN) {   // last chunk: columns past the block end contribute nothing
+          if (kv < BN) {
 #pragma unroll
             for (int i = 0; i < 32; ++i)
-              if (g * 32 + i >= kv) v[i] = SUMS ? 0u : (EPI == 0 ? 0u : 0xff800000u);   // -inf -> relu 0
-          }
-          if (p.Lout != nullptr) {
-            const int64_t li = t * BM + row;
-            if (li < p.M) {
-#pragma unroll
-              for (int i = 0; i < 32; ++i)
-                if (g * 32 + i < kv) p.Lout[li * p.K + c * BN + g * 32 + i] = __uint_as_float(v[i]);
-            }
+              if (g * 32 + i >= kv) v[i] = 0u;
           }
           if (UPDATE) {   // X for columns [col0, col0 + 32) of this row: the step
-            const int64_t li = t * BM + row;
+            const int64_t li = (int64_t)t * BM + row;
             if (li < p.M) {
               const int64_t col0 = c * BN + g * 32;
               float* mrow = p.upd_M + (p.upd_row0 + li) * RP + col0;
@@ -692,7 +983,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               if (!finite) record(p.status, NMD_ERR_DIVERGED, (int)(p.upd_row0 + li));
             }
           } else if (NEAREST) {   // columns past the set or the row itself do not count
-            const int64_t cb = c * BN + g * 32, self = t * BM + row;
+            const int64_t cb = c * BN + g * 32, self = (int64_t)t * BM + row;
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
               const float x = __uint_as_float(v[i]);
@@ -702,16 +993,13 @@ __global__ void __launch_bounds__(kThreads, 1)
               }
             }
           } else if (SUMS) {
-            const int64_t cb = c * BN + g * 32;
-            if (snext < cb + 32) {   // support columns in this group: zero them
+            uint32_t mg = 0u;
 #pragma unroll
-              for (int i = 0; i < 32; ++i) {
-                if (cb + i == snext) {
-                  v[i] = 0u;
-                  ++se;
-                  snext = se < send ? p.cidx[se] : INT64_MAX;
-                }
-              }
+            for (int w = 0; w < BN / 32; ++w) mg = w == g ? msk[w] : mg;
+            if (mg != 0u) {   // support columns in this group: zero them
+#pragma unroll
+              for (int i = 0; i < 32; ++i)
+                if ((mg >> i) & 1u) v[i] = 0u;
             }
 #pragma unroll
             for (int i = 0; i < 32; i += 2) {
@@ -720,51 +1008,55 @@ __global__ void __launch_bounds__(kThreads, 1)
               c2 = fmaf(x1, x1, c2);
               c1 += x0 + x1;
             }
-          } else if (!SPLIT) {
-            uint32_t pk[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              if (EPI == 0) {   // min(0, L)
-                pk[i] = min0_bf16x2(pack_bf16x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])));
-              } else {          // max(0, L); the MMA negates it
-                pk[i] = pack_relu_bf16x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
-                if (VOTE) nzacc |= pk[i] & 0x7fff7fffu;   // -0 counts as zero
-              }
-            }
-            tmem_st16(lcol + g * 16, pk);
-          } else {
-            // fp32-accurate: P = hi + lo, hi at columns [32 g, 32 g + 16), lo at [32 g + 16, 32 g + 32)
-            uint32_t ph[16], pl[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float x0 = __uint_as_float(v[2 * i]), x1 = __uint_as_float(v[2 * i + 1]);
-              const float e0 = EPI == 0 ? fminf(0.f, x0) : fminf(0.f, -x0);
-              const float e1 = EPI == 0 ? fminf(0.f, x1) : fminf(0.f, -x1);
-              const uint32_t hp = pack_bf16x2(e0, e1);
-              const float h0 = __uint_as_float(hp << 16), h1 = __uint_as_float(hp & 0xffff0000u);
-              ph[i] = hp;
-              pl[i] = pack_bf16x2(e0 - h0, e1 - h1);
-              if (VOTE) nzacc |= (ph[i] | pl[i]) & 0x7fff7fffu;   // -0 counts as zero
-            }
-            tmem_st16(lcol + g * 32, ph);
-            tmem_st16(lcol + g * 32 + 16, pl);
           }
         };
+        if constexpr (MODE == 0) {
+          constexpr int NG = C::HALF ? BN / 64 : BN / 32;   // this warpgroup's groups of 32 columns
+          const int g0 = C::HALF ? wg * NG : 0;
+          uint32_t va[32], vb[32];
+          if (kv < BN || p.Lout != nullptr) {
+            // a ragged last chunk (columns past the block contribute nothing),
+            // or L itself is wanted
 #pragma unroll 1
-        for (int jj = 0; jj < BN / 64; ++jj) {   // two groups per pass, both loads in flight
-          uint32_t v0[32], v1[32];
-          tmem_ld32(lcol + jj * 64, v0);
-          tmem_ld32(lcol + jj * 64 + 32, v1);
-          tmem_wait_ld(v0);
-          tmem_wait_ld(v1);
-          group(v0, 2 * jj);
-          group(v1, 2 * jj + 1);
-        }
-        if (BN % 64 != 0) {   // a last group of 32 columns
-          uint32_t v0[32];
-          tmem_ld32(lcol + (BN / 64) * 64, v0);
-          tmem_wait_ld(v0);
-          group(v0, BN / 32 - 1);
+            for (int g = g0; g < g0 + NG; ++g) {
+              tmem_ld32(lcol + g * 32, va);
+              tmem_wait_ld(va);
+              const int64_t li = (int64_t)t * BM + row;
+#pragma unroll
+              for (int i = 0; i < 32; ++i) {
+                if (g * 32 + i >= kv) va[i] = 0u;
+                else if (p.Lout != nullptr && li < p.M)   // (the bf16 mode's Z form holds -L)
+                  p.Lout[li * p.K + c * BN + g * 32 + i] =
+                      EPI == 0 && !SPLIT ? -__uint_as_float(va[i]) : __uint_as_float(va[i]);
+              }
+              to_p(va, g);
+            }
+          } else {
+            // the next group's load in flight while one is converted
+            tmem_ld32(lcol + g0 * 32, va);
+#pragma unroll
+            for (int q = 0; q < NG; q += 2) {
+              tmem_wait_ld(va);
+              if (q + 1 < NG) tmem_ld32(lcol + (g0 + q + 1) * 32, vb);
+              to_p(va, g0 + q);
+              if (q + 1 < NG) {
+                tmem_wait_ld(vb);
+                if (q + 2 < NG) tmem_ld32(lcol + (g0 + q + 2) * 32, va);
+                to_p(vb, g0 + q + 1);
+              }
+            }
+          }
+        } else {
+#pragma unroll 1
+          for (int jj = 0; jj < BN / 64; ++jj) {   // two groups per pass, both loads in flight
+            uint32_t v0[32], v1[32];
+            tmem_ld32(lcol + jj * 64, v0);
+            tmem_ld32(lcol + jj * 64 + 32, v1);
+            tmem_wait_ld(v0);
+            tmem_wait_ld(v1);
+            group(v0, 2 * jj);
+            group(v1, 2 * jj + 1);
+          }
         }
         if (LOSS) {
           if (SUMS) {
@@ -777,17 +1069,22 @@ __global__ void __launch_bounds__(kThreads, 1)
         } else {
           if (VOTE) {   // published before the arrive (release) that MMA2 acquires
             const bool nz = __any_sync(0xffffffffu, nzacc != 0u);
-            if (lane == 0) pflag[4 * lb + (warp & 3)] = nz ? 1u : 0u;
+            if (lane == 0) pflag[8 * lb + (C::HALF ? warp : (warp & 3))] = nz ? 1u : 0u;
           }
           tmem_wait_st();
           fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(b_pfull + 8 * lb);
+          // the previous tile's R, after this warpgroup's first chunk of the tile
+          if (C::NRB == 2 && pend >= 0) {
+            if (!(ok = readout(pend, tt - 1))) break;
+            pend = -1;
+          }
         }
       }
       if (!ok) break;
       if (NEAREST) {   // this warpgroup's best of the row; the two are merged by atomicMax
-        const int64_t li = t * BM + row;
+        const int64_t li = (int64_t)t * BM + row;
         if (li < p.M && nidx >= 0) {
           const uint32_t b = __float_as_uint(nbest);
           const uint32_t ord = (b & 0x80000000u) ? ~b : (b | 0x80000000u);   // float order as unsigned
@@ -796,48 +1093,22 @@ __global__ void __launch_bounds__(kThreads, 1)
         nbest = -INFINITY;
         nidx = -1;
       }
-      if (!LOSS) {
-        if (!(ok = warp_wait(b_rfull, (uint32_t)(tt & 1), abort_flag, p.status, 8))) break;
-        fence_after();
-        const int64_t li = t * BM + row;
-        float* dst = Rout + li * RP + (C::RHALF ? (int64_t)blockIdx.y * C::NR : 0);
-        constexpr int NJ = (C::NR + 31) / 32;
-#pragma unroll 1
-        for (int j = wg; j < NJ; j += 2) {
-          // the warp's last TMEM read of the tile releases R (MMA2 may start
-          // the next tile) before the adds and global stores
-          const bool last = j + 2 >= NJ;
-          uint32_t v[32];
-          tmem_ld32(tmem + lane_base + C::COL_R + j * 32, v);   // RP = 16 reads 16 columns past R
-          tmem_wait_ld(v);
-          if (last) {
-            fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(b_rempty);
-          }
-          if (li < p.M) {
-#pragma unroll
-            for (int i = 0; i < 32; i += 4)
-              if (j * 32 + i < C::NR)
-                *(float4*)(dst + j * 32 + i) = make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]),
-                                                          __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
-          }
-        }
-        if (wg >= NJ) {   // no columns for this warpgroup (r_pad = 16): release at once
-          fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(b_rempty);
-        }
-      }
       // refill this tile's W buffer with the tile NWB steps ahead
-      const int64_t tn = t + (int64_t)NWB * gridDim.x;
-      if (!C::WSMEM && tn < ntiles) {
-        const int wb = (int)(tt % NWB);
-        if (!(ok = warp_wait(b_wempty + 8 * wb, (uint32_t)((tt / NWB) & 1), abort_flag, p.status, 9))) break;
+      const int tn = t + NWB * (int)gridDim.x;
+      if (!C::WSMEM && tn < (int)ntiles) {
+        const int wb = tt % NWB;
+        if (!(ok = conv_wait(b_wempty + 8 * wb, (uint32_t)((tt / NWB) & 1), abort_flag, p.status, 9))) break;
         fence_after();
         load_w(tn, wb);
       }
+      if (!LOSS) {
+        // (a tile in which this warpgroup had no chunk has not read the previous R yet)
+        if (C::NRB == 2 && pend >= 0 && !(ok = readout(pend, tt - 1))) break;
+        if (C::NRB == 2) pend = t;
+        else if (!(ok = readout(t, tt))) break;
+      }
     }
+    if (!LOSS && C::NRB == 2 && ok && pend >= 0) readout(pend, tt - 1);
     if (SUMS) {
       // fixed-order reduction over the 256 epilogue threads
       red[2 * et] = s2;
@@ -925,7 +1196,7 @@ bool tensor_map(const bf16* base, int64_t rows, int rp, int panel_w, int bn, CUt
 
 template <int RP, int EPI, bool SPLIT, int MODE, int SKIPM = 0>
 nmd_status run(const Factor& fm, const Factor& fq, const TcParams& p, int grid, cudaStream_t s) {
-  using C = Cfg<RP, SPLIT, MODE != 0>;
+  using C = Cfg<RP, SPLIT, MODE != 0, SKIPM != 0>;
   CUtensorMap th, tl, tl2;
   if (!tensor_map(fq.hi, fq.rows, RP, C::PANEL_W, C::BN, &th)) return NMD_ERR_CUDA;
   if (!tensor_map(fq.lo, fq.rows, RP, C::PANEL_W, C::BN, &tl)) return NMD_ERR_CUDA;
@@ -994,14 +1265,15 @@ nmd_status dispatch(int rp, int epilogue, bool split, const Factor& fm, const Fa
 
 }  // namespace
 
+// (of the chunk-skipping kernels)
 int panel_chunk_rows(int rp, int precision) {
   const bool split = precision == NMD_FP32;
   switch (rp) {
-    case 16: return split ? Cfg<16, true, false>::BN : Cfg<16, false, false>::BN;
-    case 32: return split ? Cfg<32, true, false>::BN : Cfg<32, false, false>::BN;
-    case 64: return split ? Cfg<64, true, false>::BN : Cfg<64, false, false>::BN;
-    case 128: return split ? Cfg<128, true, false>::BN : Cfg<128, false, false>::BN;
-    default: return split ? Cfg<256, true, false>::BN : Cfg<256, false, false>::BN;
+    case 16: return split ? Cfg<16, true, false, true>::BN : Cfg<16, false, false, true>::BN;
+    case 32: return split ? Cfg<32, true, false, true>::BN : Cfg<32, false, false, true>::BN;
+    case 64: return split ? Cfg<64, true, false, true>::BN : Cfg<64, false, false, true>::BN;
+    case 128: return split ? Cfg<128, true, false, true>::BN : Cfg<128, false, false, true>::BN;
+    default: return split ? Cfg<256, true, false, true>::BN : Cfg<256, false, false, true>::BN;
   }
 }
 
@@ -1065,17 +1337,20 @@ void launch_wait_selftest(int* status, uint64_t limit_ns, cudaStream_t s) {
 }
 
 nmd_status launch_update_tc(const StepArgs& a, const float* R, const float* Rs, const uint8_t* flags,
-                            const Factor& gi, float eta, float gamma, bool momentum, int* status, int num_sms,
-                            cudaStream_t s) {
+                            const Factor& gi, float eta, float gamma, bool momentum, int* status, cudaStream_t s) {
   if (a.M <= 0) return NMD_OK;
   TcParams p{0, a.M, 0, a.rp, nullptr, nullptr, nullptr, nullptr, status, nullptr, nullptr, nullptr, nullptr, 0,
              0, 0, nullptr, 0, nullptr, R, Rs, flags, a.fm->master, a.fm->E, a.fm->hi, a.m0, eta, gamma,
              momentum ? 1 : 0, a.epilogue == NMD_EPI_DELTA ? 1 : 0};
+  // One tile per CTA: a deferred update shares the GPU with the next step's
+  // dense kernel, on the SMs its grid leaves free, and CTAs that retire every
+  // few microseconds let the next step's G^{-1} kernel (higher priority, 188 KB
+  // of shared memory) have one of those SMs.  With persistent CTAs it waited
+  // for the whole deferred update: 583 us for the Gram chain of a 69,627-row
+  // step against 311 us of dense kernel.
   const int64_t ntiles = (a.M + BM - 1) / BM;
-  const int64_t rounds = (ntiles + num_sms - 1) / num_sms;
-  const int grid = (int)((ntiles + rounds - 1) / rounds);
   if (a.rp != 256) return NMD_ERR_UNSUPPORTED;
-  return run<256, 0, true, 3>(*a.fm, gi, p, grid, s);
+  return run<256, 0, true, 3>(*a.fm, gi, p, (int)ntiles, s);
 }
 
 nmd_status launch_nearest_tc(const Factor& f, int64_t N, int rp, unsigned long long* keys, int* status,
