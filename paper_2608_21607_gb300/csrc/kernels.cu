@@ -1454,64 +1454,82 @@ __global__ void __launch_bounds__(256, (RP <= 64 ? 3 : 1)) update_kernel(float* 
 // entry (SUBTRACT: the CUDA-core loss pass), Shat^2 and Shat are subtracted
 // again here, with L formed by the same sequential fma chain as that pass so
 // the two cancel exactly.  The tensor-core loss pass skips support entries,
-// and nothing is subtracted.  One warp per row of S, fp64 sums.
+// and nothing is subtracted.
+//
+// What bounds it: the gathers of the B rows (from L2).  The entries, not the
+// rows, are cut into equal ranges, one per warp: a power-law graph has rows of
+// up to n entries, and with a warp per row the longest row set the time
+// (139,255 nodes, 2.8M entries, r = 64: 38 - 70 ms of a loss call).  A warp
+// takes 32 entries at a time: each lane finds its entry's row by a binary
+// search over the warp's rows; eight lanes form a dot product, four entries at
+// once, and pass it to the entry's lane, so that the fp64 terms (a few per
+// cycle and SM on this chip) are formed for 32 entries by one instruction.
+// The fp32 products are summed as a 32-lane butterfly over the columns would
+// (c + 16, c + 8, 4, 2, 1).
 // ---------------------------------------------------------------------------
-template <int VPL, bool SUBTRACT>
+template <int RP, bool SUBTRACT>
 __global__ void __launch_bounds__(256) loss_sparse_kernel(const int64_t* __restrict__ rowptr,
                                                           const int32_t* __restrict__ col,
-                                                          const float* __restrict__ val, int64_t m,
+                                                          const float* __restrict__ val, int64_t m, int64_t nnz,
                                                           const float* __restrict__ Wop,
-                                                          const float* __restrict__ Bop, int rp,
+                                                          const float* __restrict__ Bop,
                                                           double* __restrict__ parts) {
+  constexpr int CV = RP >= 32 ? RP / 32 : 1;   // columns of a lane at distance 32
+  constexpr int CK = RP >= 32 ? 4 : RP / 8;    // 8-column steps within 32 columns
   __shared__ double red[8][4];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, sub = lane & 7;
   double sa = 0, sb = 0, smn = 0, smx = 0;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < m; i += nw) {
-    float wv[VPL];
-#pragma unroll
-    for (int v = 0; v < VPL; ++v) {
-      const int c = lane + 32 * v;
-      wv[v] = c < rp ? __ldg(Wop + i * rp + c) : 0.f;
+  const int64_t per = ((nnz + nw - 1) / nw + 31) / 32 * 32;
+  const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int64_t eb = w * per, ee = eb + per < nnz ? eb + per : nnz;
+  // the row of entry e: the last row i of [lo, hi] with rowptr[i] <= e
+  auto row_of = [&](int64_t e, int lo, int hi) {
+    while (lo < hi) {
+      const int mid = (int)(((int64_t)lo + hi + 1) >> 1);
+      if (__ldg(rowptr + mid) <= e) lo = mid;
+      else hi = mid - 1;
     }
-    for (int64_t e0 = rowptr[i]; e0 < rowptr[i + 1]; e0 += 32) {
-      // lane l takes entry e0 + l
+    return lo;
+  };
+  if (eb < ee) {
+    int rlo = row_of(eb, 0, (int)(m - 1));
+    const int rhi = row_of(ee - 1, rlo, (int)(m - 1));
+    for (int64_t e0 = eb; e0 < ee; e0 += 32) {
       const int64_t e = e0 + lane;
-      const bool live = e < rowptr[i + 1];
+      const bool live = e < ee;
+      const int row = row_of(live ? e : ee - 1, rlo, rhi);   // (a row past the last entry repeats its row)
+      const int cj = __ldg(col + (live ? e : ee - 1));
+      rlo = __shfl_sync(0xffffffffu, row, 31);
+      float L = 0.f;
       if (SUBTRACT) {
-        if (live) {
-          const int64_t j = col[e];
-          float L = 0.f;
-          for (int c = 0; c < rp; ++c) L = fmaf(__ldg(Wop + i * rp + c), __ldg(Bop + j * rp + c), L);
-          const double Ld = L, S = val[e];
-          const double sh = Ld > 0 ? Ld : 0.0;
-          sa += (S - Ld) * (S - Ld) - sh * sh;
-          sb += (S - sh) * (S - sh) - sh * sh;
-          smn += S < sh ? S : sh;
-          smx += (S > sh ? S : sh) - sh;
-        }
+        for (int c = 0; c < RP; ++c)
+          L = fmaf(__ldg(Wop + (int64_t)row * RP + c), __ldg(Bop + (int64_t)cj * RP + c), L);
       } else {
-        const int64_t rem = rowptr[i + 1] - e0;
-        const int cnt = rem < 32 ? (int)rem : 32;
-        for (int q = 0; q < cnt; ++q) {
-          const int64_t j = col[e0 + q];
-          float part = 0.f;
+#pragma unroll 2
+        for (int it = 0; it < 8; ++it) {
+          const int src = it * 4 + (lane >> 3);
+          const float* wr = Wop + (int64_t)__shfl_sync(0xffffffffu, row, src) * RP + sub;
+          const float* br = Bop + (int64_t)__shfl_sync(0xffffffffu, cj, src) * RP + sub;
+          float q[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-          for (int v = 0; v < VPL; ++v) {
-            const int c = lane + 32 * v;
-            part = fmaf(wv[v], c < rp ? __ldg(Bop + j * rp + c) : 0.f, part);
-          }
+          for (int v = 0; v < CV; ++v)
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-          if (lane == q) {
-            const double Ld = part, S = val[e0 + q];
-            const double sh = Ld > 0 ? Ld : 0.0;
-            sa += (S - Ld) * (S - Ld);
-            sb += (S - sh) * (S - sh);
-            smn += S < sh ? S : sh;
-            smx += S > sh ? S : sh;
-          }
+            for (int k = 0; k < CK; ++k) q[k] = fmaf(__ldg(wr + 32 * v + 8 * k), __ldg(br + 32 * v + 8 * k), q[k]);
+          float part = (q[0] + q[2]) + (q[1] + q[3]);
+#pragma unroll
+          for (int o = 4; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+          const float mine = __shfl_sync(0xffffffffu, part, (lane & 3) * 8);
+          if ((lane >> 2) == it) L = mine;
         }
+      }
+      if (live) {
+        const double Ld = L, S = __ldg(val + e);
+        const double sh = Ld > 0 ? Ld : 0.0;
+        sa += (S - Ld) * (S - Ld) - (SUBTRACT ? sh * sh : 0.0);
+        sb += (S - sh) * (S - sh) - (SUBTRACT ? sh * sh : 0.0);
+        smn += S < sh ? S : sh;
+        smx += (S > sh ? S : sh) - (SUBTRACT ? sh : 0.0);
       }
     }
   }
@@ -1528,7 +1546,7 @@ __global__ void __launch_bounds__(256) loss_sparse_kernel(const int64_t* __restr
   __syncthreads();
   if (threadIdx.x < 4) {
     double s = 0;
-    for (int w = 0; w < 8; ++w) s += red[w][threadIdx.x];
+    for (int k = 0; k < 8; ++k) s += red[k][threadIdx.x];
     parts[(size_t)blockIdx.x * 8 + threadIdx.x] = s;
   }
 }
@@ -1974,20 +1992,21 @@ void launch_combine(float* R, const float* Rs, const uint8_t* flags, int64_t row
 void launch_loss_sparse(const nmd_handle* h, double* parts, int nparts, cudaStream_t s) {
   // fp32 masters in every precision, like the support correction of the update
   const bool subtract = h->opt.precision == NMD_SIMT;
-#define NMD_LS(V)                                                                                          \
-  do {                                                                                                     \
-    if (subtract)                                                                                          \
-      loss_sparse_kernel<V, true><<<nparts, 256, 0, s>>>(h->ws.rowptr, h->ws.col, h->ws.val, h->m,           \
-                                                        h->W.master, h->B.master, h->rp, parts);           \
-    else                                                                                                   \
-      loss_sparse_kernel<V, false><<<nparts, 256, 0, s>>>(h->ws.rowptr, h->ws.col, h->ws.val, h->m,          \
-                                                         h->W.master, h->B.master, h->rp, parts);          \
+#define NMD_LS(RPV)                                                                                              \
+  do {                                                                                                           \
+    if (subtract)                                                                                                \
+      loss_sparse_kernel<RPV, true><<<nparts, 256, 0, s>>>(h->ws.rowptr, h->ws.col, h->ws.val, h->m, h->nnz,      \
+                                                           h->W.master, h->B.master, parts);                     \
+    else                                                                                                         \
+      loss_sparse_kernel<RPV, false><<<nparts, 256, 0, s>>>(h->ws.rowptr, h->ws.col, h->ws.val, h->m, h->nnz,     \
+                                                            h->W.master, h->B.master, parts);                    \
   } while (0)
   switch (h->rp) {
-    case 16: case 32: NMD_LS(1); break;
-    case 64: NMD_LS(2); break;
-    case 128: NMD_LS(4); break;
-    default: NMD_LS(8); break;
+    case 16: NMD_LS(16); break;
+    case 32: NMD_LS(32); break;
+    case 64: NMD_LS(64); break;
+    case 128: NMD_LS(128); break;
+    default: NMD_LS(256); break;
   }
 #undef NMD_LS
 }
