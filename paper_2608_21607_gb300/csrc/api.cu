@@ -748,15 +748,28 @@ nmd_status run_step_roles(nmd_handle* h, const Roles& ro, int kind, bool do_upda
   const bool rows64 = (ro.K + 63) / 64 <= kGramParts;
   const int nparts = rows64 ? (int)((ro.K + 63) / 64) : kGramParts;
   const int64_t chunk = rows64 ? 64 : ((ro.K + nparts - 1) / nparts + 31) / 32 * 32;
+  // At r_pad >= 128 a dense CTA leaves no room on its SM for a Gram block: the
+  // partials run ahead of the dense kernel on the main stream (17 us at r =
+  // 256, 8,192 rows) instead of on the few SMs the dense grid leaves free,
+  // where they took longer than the dense kernel.
+  const bool gram_first = need_gram && h->rp >= 128;
+  if (gram_first) {
+    TimedScope ts(h, NMD_K_GRAM, s);
+    launch_gram_parts(ro.fq, rounded, ro.q0, ro.K, h->rp, h->ws.gram_part, nparts, chunk, s);
+    h->launches++;
+  }
   CK(h, cudaEventRecord(h->ev_fork, s));
   CK(h, cudaStreamWaitEvent(h->side, h->ev_fork, 0));
   CK(h, cudaStreamWaitEvent(h->side2, h->ev_fork, 0));
   if (need_gram) {
     TimedScope ts(h, NMD_K_GRAM, h->side);
-    launch_gram(ro.fq, rounded, ro.q0, ro.K, h->r, h->rp, h->ws.gram_part, nparts, chunk, (float)h->opt.ridge, G,
-                h->side);
+    if (!gram_first) {
+      launch_gram_parts(ro.fq, rounded, ro.q0, ro.K, h->rp, h->ws.gram_part, nparts, chunk, h->side);
+      h->launches++;
+    }
+    launch_gram_reduce(h->ws.gram_part, nparts, h->r, h->rp, (float)h->opt.ridge, G, h->side);
     launch_chol_inv(G, h->r, h->rp, Ginv, gsplit_of(h, Ginv), h->ws.status, h->side);
-    h->launches += 3;
+    h->launches += 2;
     if (tc_update(h)) {   // the pieces of G^{-1} for the tensor-core update
       Factor gi = *gi_of(h, Ginv);
       launch_pack(Ginv, false, h->rp, h->rp, h->rp, gi, h->side);
@@ -1016,8 +1029,12 @@ nmd_status nmd_create(int64_t m, int64_t n, int32_t r, const int64_t* row_ptr,
   int least = 0, greatest = 0;
   e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
   const int side_prio = greatest < least ? greatest + 1 : greatest;
+  // the Gram chain before the support term: its three short kernels wait for
+  // SM room one after the other (planted 20,000^2, r = 32: 62 -> 37 us beside
+  // the support kernel, which takes 50 us either way)
+  const int side2_prio = std::min(side_prio + 1, least);
   if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, side_prio);
-  if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->side2, cudaStreamNonBlocking, side_prio);
+  if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->side2, cudaStreamNonBlocking, side2_prio);
   if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->hp, cudaStreamNonBlocking, greatest);
   if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->aux, cudaStreamNonBlocking, least);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming);

@@ -451,7 +451,7 @@ template <int RP>
 struct TileChol {
   static constexpr int TB = 32, NT = RP / TB, LDT = TB + 1, TSZ = TB * LDT;
   static constexpr int NTILE = NT * (NT + 1) / 2;
-  static constexpr int NTHR = RP * 4 > 1024 ? 1024 : RP * 4;
+  static constexpr int NTHR = RP * 4 > 512 ? 512 : RP * 4;
   static constexpr int PBUF = TB * RP;   // the transposed panel (32 x RP), or the T_IJ of one tile row
   static constexpr size_t SMEM = ((size_t)NTILE * TSZ + PBUF + 3 * RP) * sizeof(float);
   static_assert(RP % TB == 0 && NT >= 2, "tile form for r_pad >= 64");
@@ -466,8 +466,12 @@ __device__ __forceinline__ void tile_of(int q, int& I, int& J) {
   J = q - ((I * (I + 1)) >> 1);
 }
 
+// (registers capped at 64: beside a dense CTA of r_pad = 64 there are 20,480 left
+// on an SM, which 256 threads of 128 did not fit into, so that the inverse waited
+// for an SM without a dense CTA: 105 -> 78 us for the Gram chain beside it; at
+// r_pad = 256 512 threads of 64 find room beside the support term's blocks)
 template <int RP>
-__global__ void __launch_bounds__(TileChol<RP>::NTHR, 1) ldlt_inv_tile_kernel(const float* __restrict__ G, int r,
+__global__ void __launch_bounds__(1024, 1) ldlt_inv_tile_kernel(const float* __restrict__ G, int r,
                                                                           float* __restrict__ Ginv,
                                                                           bf16* __restrict__ gsplit,
                                                                           int* __restrict__ status) {
@@ -1586,15 +1590,24 @@ void launch_unpack(const float* master, bool dst_is_rxN, int64_t N, int r, int r
   unpack_kernel<<<grid_for(N * r, 256), 256, 0, s>>>(master, dst_is_rxN, N, r, rp, dst);
 }
 
-void launch_gram(const Factor* fq, bool rounded, int64_t q0, int64_t K, int r, int rp, float* parts, int nparts,
-                 int64_t chunk, float ridge, float* G, cudaStream_t s) {
+void launch_gram_parts(const Factor* fq, bool rounded, int64_t q0, int64_t K, int rp, float* parts, int nparts,
+                       int64_t chunk, cudaStream_t s) {
   int nt = (rp + 63) / 64;
   dim3 grid(nt * (nt + 1) / 2, nparts);
   if (rounded)
     gram_kernel<bf16><<<grid, 256, 0, s>>>(fq->hi, q0, K, rp, parts, chunk);
   else
     gram_kernel<float><<<grid, 256, 0, s>>>(fq->master, q0, K, rp, parts, chunk);
+}
+
+void launch_gram_reduce(const float* parts, int nparts, int r, int rp, float ridge, float* G, cudaStream_t s) {
   gram_reduce_kernel<<<(unsigned)((rp * rp + 255) / 256), 256, 0, s>>>(parts, nparts, r, rp, ridge, G);
+}
+
+void launch_gram(const Factor* fq, bool rounded, int64_t q0, int64_t K, int r, int rp, float* parts, int nparts,
+                 int64_t chunk, float ridge, float* G, cudaStream_t s) {
+  launch_gram_parts(fq, rounded, q0, K, rp, parts, nparts, chunk, s);
+  launch_gram_reduce(parts, nparts, r, rp, ridge, G, s);
 }
 
 void launch_small_gemm(const float* A, int64_t lda, const float* B, int64_t ldb, float* C, int64_t ldc, int64_t M,

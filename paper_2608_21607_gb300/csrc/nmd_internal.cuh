@@ -240,6 +240,10 @@ void launch_unpack(const float* master, bool dst_is_rxN, int64_t N, int r, int r
 // G = Q^T Q of the Q-side rows [q0, q0 + K) (+ ridge on the diagonal) via
 // nparts fixed-order partials of `chunk` rows; rounded: of their bf16 pieces
 // (hi) instead of the fp32 masters.
+void launch_gram_parts(const Factor* fq, bool rounded, int64_t q0, int64_t K, int rp, float* parts, int nparts,
+                       int64_t chunk, cudaStream_t s);
+void launch_gram_reduce(const float* parts, int nparts, int r, int rp, float ridge, float* G, cudaStream_t s);
+// both
 void launch_gram(const Factor* fq, bool rounded, int64_t q0, int64_t K, int r, int rp, float* parts, int nparts,
                  int64_t chunk, float ridge, float* G, cudaStream_t s);
 // Ginv = G^{-1} through the Cholesky (L D L^T) factorisation; NMD_ERR_NOT_SPD
