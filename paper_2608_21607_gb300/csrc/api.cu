@@ -647,6 +647,14 @@ nmd_status launch_update_rows(nmd_handle* h, const StepArgs& a, const Roles& ro,
                               const uint8_t* flags, const float* Ginv, int64_t lo, int64_t hi, bool momentum,
                               cudaStream_t s) {
   if (hi <= lo) return NMD_OK;
+  if (update_takes_ranges(a, gsplit_of(h, Ginv))) {
+    TimedScope ts(h, NMD_K_UPDATE, s);
+    if (!launch_update_ranges(a, 0, lo, hi - lo, R, Rs, flags, gsplit_of(h, Ginv), (float)h->opt.eta,
+                              momentum ? (float)h->opt.gamma : 0.f, momentum, nullptr, h->ws.status, s))
+      return fail(h, NMD_ERR_CUDA, "update kernel");
+    h->launches++;
+    return NMD_OK;
+  }
   StepArgs sub = a;
   sub.m0 = ro.m0 + lo;
   sub.M = hi - lo;
@@ -821,8 +829,17 @@ nmd_status run_step_roles(nmd_handle* h, const Roles& ro, int kind, bool do_upda
     if (lo > 0 || hi < ro.M) {
       CK(h, cudaEventRecord(h->ev_prio, s));
       CK(h, cudaStreamWaitEvent(h->aux, h->ev_prio, 0));
-      if ((st = launch_update_rows(h, a, ro, R, Rs, flags, Ginv, 0, lo, momentum, h->aux)) != NMD_OK) return st;
-      if ((st = launch_update_rows(h, a, ro, R, Rs, flags, Ginv, hi, ro.M, momentum, h->aux)) != NMD_OK) return st;
+      if (update_takes_ranges(a, gsplit_of(h, Ginv))) {   // both ranges in one launch
+        TimedScope ts(h, NMD_K_UPDATE, h->aux);
+        if (!launch_update_ranges(a, lo, hi, ro.M - hi, R, Rs, flags, gsplit_of(h, Ginv), (float)h->opt.eta,
+                                  momentum ? (float)h->opt.gamma : 0.f, momentum, h->ws.counters + 2, h->ws.status,
+                                  h->aux))
+          return fail(h, NMD_ERR_CUDA, "deferred update kernel");
+        h->launches++;
+      } else {
+        if ((st = launch_update_rows(h, a, ro, R, Rs, flags, Ginv, 0, lo, momentum, h->aux)) != NMD_OK) return st;
+        if ((st = launch_update_rows(h, a, ro, R, Rs, flags, Ginv, hi, ro.M, momentum, h->aux)) != NMD_OK) return st;
+      }
       nmd_handle::Pending& pm = h->pend[fm];
       CK(h, cudaEventRecord(pm.ev, h->aux));
       pm.active = true;

@@ -729,8 +729,12 @@ __device__ __forceinline__ void load16(float* f, const float* p) {
   f[0] = v.x; f[1] = v.y; f[2] = v.z; f[3] = v.w;
 }
 
+// Blocks of 128 threads (of 64 registers): beside a dense CTA and an update block
+// of r_pad = 64 an SM sub-partition has 2,048 registers left, one warp's.
+constexpr int kSparseThreads = 128;
+
 template <int RP, typename T>
-__global__ void __launch_bounds__(256, 4) sparse_group_kernel(const PanelRow* __restrict__ rows, int64_t nrows,
+__global__ void __maxnreg__(RP == 64 ? 56 : 64) sparse_group_kernel(const PanelRow* __restrict__ rows, int64_t nrows,
                                                            const T* __restrict__ Mop, int64_t m0,
                                                            const T* __restrict__ Qop,
                                                            const int32_t* __restrict__ qidx,
@@ -841,7 +845,7 @@ __device__ __forceinline__ void stage16(float* dst, const bf16* src) {
 }
 
 template <int LPE, int CPL, typename T>
-__global__ void __launch_bounds__(256, 2) sparse_long_kernel(const PanelRow* __restrict__ segs, int64_t nseg,
+__global__ void __launch_bounds__(kSparseThreads, 4) sparse_long_kernel(const PanelRow* __restrict__ segs, int64_t nseg,
                                                           const T* __restrict__ Mop, int64_t m0,
                                                           const T* __restrict__ Qop,
                                                           const int32_t* __restrict__ qidx,
@@ -853,11 +857,11 @@ __global__ void __launch_bounds__(256, 2) sparse_long_kernel(const PanelRow* __r
   constexpr int NPF = 4;                       // entry iterations whose indices are fetched together
   constexpr int VEC = 16 / (int)sizeof(T);     // elements per 16-byte load
   constexpr int LPC = CPL / VEC;               // 16-byte loads per 32-column chunk
-  __shared__ __align__(16) float stage[8][32 * CS];
+  __shared__ __align__(16) float stage[kSparseThreads / 32][32 * CS];
   const int lane = threadIdx.x & 31;
   const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   if (w >= nseg) return;
-  float* buf = stage[(threadIdx.x >> 5) & 7];
+  float* buf = stage[threadIdx.x >> 5];
   const PanelRow pr = segs[w];
   const int sub = lane % LPE, slot = lane / LPE;
   const int64_t i = pr.row;
@@ -963,6 +967,8 @@ __global__ void __launch_bounds__(256) sparse_reduce_kernel(const PanelRow* __re
 // In the bf16 mode R and Ginv belong to the bf16-rounded Q-side rows (R = Z Qt,
 // Ginv = (Qt^T Qt)^{-1}), so X is the least-squares solution for them.
 // Skipped entirely while a sticky error is set.
+// (The bf16 mode at r_pad <= 64 has its own kernel, update_tc_kernel below, at
+// 256 the update pass of the dense kernel.)
 // X = R G^{-1} is a small GEMM per tile of TR rows.  A block keeps CW columns
 // of G^{-1} in shared memory; the tile's R rows (contiguous in global memory)
 // are copied into a double buffer with cp.async one tile ahead, and each
@@ -1451,6 +1457,219 @@ __global__ void __launch_bounds__(256, (RP <= 64 ? 3 : 1)) update_kernel(float* 
 }
 
 // ---------------------------------------------------------------------------
+// The same update in the bf16 mode at r_pad <= 64: X = (R + Rs) G^{-1} on the
+// tensor cores (mma.sync, R + Rs and G^{-1} as hi + lo bf16 pieces, three
+// products, fp32 accumulation), as blocks that walk over tiles of TR rows.
+// What bounds it: bytes in flight.  A deferred update runs beside the dense
+// kernel, which leaves room for one block of 72 registers per SM sub-partition
+// pair and about 60 KB of shared memory; a block per tile loads, computes and
+// stores one after the other there (137 us for 135,000 rows of r_pad = 64
+// beside a dense kernel of 103 us, which the next step but one then waits for).
+// Here, at r_pad = 64, one block per SM takes tiles from a counter, with the R, M
+// and E rows of the next tile on their way (cp.async, two stages) while one is
+// computed, and keeps its warps' columns of G^{-1} in registers: 115 us for both
+// row ranges, and 9 instead of 15 us for the 4,096 rows on the critical path.
+// Rows: [0, n0) and [r1, r1 + n1) of the step's M side (the second range is
+// empty, or the rows behind those updated first); tiles do not cross ranges.
+// counter: nullptr = block b takes tile b only (the grid covers the tiles);
+// else the next tile, zero at launch, handed out by atomicAdd.
+// ---------------------------------------------------------------------------
+template <int RP>
+struct UpdTc {
+  static constexpr int TR = RP == 64 ? 32 : 64;      // rows per tile
+  static constexpr int RG = TR / 16;                 // 16-row groups of warps
+  static constexpr int WC = RP / (8 / RG);           // columns per warp
+  static constexpr int NT = WC / 8;                  // 8-column tiles per warp
+  static constexpr int SR = RP + 8;                  // row stride of a staged R tile (floats)
+  static constexpr int SB = split_stride(RP);
+  static constexpr int NV = TR * RP / 4 / 256;       // 16-byte pieces of a tile per thread
+  static constexpr int STAGE = TR * SR + 2 * TR * RP;   // floats: R, M, E
+  static constexpr size_t SMEM = 2 * (size_t)STAGE * sizeof(float);
+  static_assert(WC >= 8 && NV >= 1, "tiling");
+};
+
+template <int RP>
+__global__ void __maxnreg__(RP == 64 ? 72 : 64) update_tc_kernel(float* __restrict__ M, bf16* __restrict__ Mhi,
+                                                         float* __restrict__ E, int64_t m0, int64_t n0, int64_t r1,
+                                                         int64_t n1, const float* __restrict__ R,
+                                                         const float* __restrict__ Rs,
+                                                         const uint8_t* __restrict__ flags,
+                                                         const bf16* __restrict__ gsplit, float eta, float gamma,
+                                                         int momentum, int delta_form, int* __restrict__ counter,
+                                                         int* __restrict__ status) {
+  using C = UpdTc<RP>;
+  constexpr int TR = C::TR, SR = C::SR, SB = C::SB, NV = C::NV, NT = C::NT, KS = RP / 16;
+  extern __shared__ __align__(16) float sm[];
+  __shared__ int next_batch;
+  if (*(volatile int*)status != 0) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t t0 = (n0 + TR - 1) / TR, ntiles = t0 + (n1 + TR - 1) / TR;
+  // first row (relative to the step's M side) and row count of a tile
+  auto rows_of = [&](int64_t t, int64_t& row) -> int {
+    const bool a = t < t0;
+    const int64_t i = (a ? t : t - t0) * TR, left = (a ? n0 : n1) - i;
+    row = a ? i : r1 + i;
+    return (int)(left < TR ? left : TR);
+  };
+  // copy a tile's R, M and E rows into stage b; this thread's pieces of Rs
+  auto issue = [&](int64_t t, int b) {
+    int64_t row;
+    const int nr = rows_of(t, row);
+    float* st = sm + b * C::STAGE;
+#pragma unroll
+    for (int u = 0; u < NV; ++u) {
+      const int e = tid + 256 * u, i = 4 * e / RP, c = 4 * e % RP;
+      if (i < nr) {
+        cp_async16(st + i * SR + c, R + (row + i) * RP + c);
+        cp_async16(st + TR * SR + 4 * e, M + (m0 + row + i) * RP + c);
+        if (momentum) cp_async16(st + TR * SR + TR * RP + 4 * e, E + (m0 + row + i) * RP + c);
+      }
+    }
+  };
+  // the flags of this thread's pieces of a tile, and the flagged pieces of Rs
+  auto load_flags = [&](int64_t t, int(&f)[NV]) {
+#pragma unroll
+    for (int u = 0; u < NV; ++u) f[u] = 0;
+    if (t >= ntiles) return;
+    int64_t row;
+    const int nr = rows_of(t, row);
+#pragma unroll
+    for (int u = 0; u < NV; ++u) {
+      const int i = 4 * (tid + 256 * u) / RP;
+      if (i < nr) f[u] = __ldg(flags + row + i);
+    }
+  };
+  auto load_rs = [&](int64_t t, const int(&f)[NV], float4(&sv)[NV]) {
+    int64_t row;
+    rows_of(t, row);
+#pragma unroll
+    for (int u = 0; u < NV; ++u) {
+      const int e = tid + 256 * u, i = 4 * e / RP, c = 4 * e % RP;
+      sv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (f[u]) sv[u] = *(const float4*)(Rs + (row + i) * RP + c);
+    }
+  };
+  // the tile, the next one and the one after that: batches of four tiles, the
+  // first by block index, the others drawn from the counter two tiles and
+  // more before they are needed
+  int64_t t = counter ? 4 * (int64_t)blockIdx.x : blockIdx.x;
+  if (t >= ntiles) return;
+  int64_t t1 = counter ? t + 1 : ntiles, t2 = counter ? t + 2 : ntiles;
+  float4 sv[NV];
+  int f[NV];
+  issue(t, 0);
+  cp_async_commit();
+  load_flags(t, f);
+  int drawn = 0;
+  if (counter && tid == 0) next_batch = atomicAdd(counter, 1) + (int)gridDim.x;
+  load_rs(t, f, sv);
+  load_flags(t1, f);
+  // this warp's 16 rows of a tile (r0) and its columns of G^{-1} (n0w): the B
+  // fragments of every k step, both pieces
+  const int g = lane / 4, c2 = 2 * (lane % 4);
+  const int r0 = 16 * (warp % C::RG), nw = (warp / C::RG) * C::WC;
+  uint32_t bh[KS][NT][2], bl[KS][NT][2];
+#pragma unroll
+  for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+      const bf16* src = gsplit + (nw + 8 * n + g) * SB + 16 * ks + c2;
+      bh[ks][n][0] = __ldg(reinterpret_cast<const uint32_t*>(src));
+      bh[ks][n][1] = __ldg(reinterpret_cast<const uint32_t*>(src + 8));
+      bl[ks][n][0] = __ldg(reinterpret_cast<const uint32_t*>(src + RP * SB));
+      bl[ks][n][1] = __ldg(reinterpret_cast<const uint32_t*>(src + RP * SB + 8));
+    }
+  for (int b = 0;; b ^= 1) {
+    // the next tile's rows on their way
+    const bool more = t1 < ntiles;
+    if (more) issue(t1, b ^ 1);
+    cp_async_commit();
+    cp_async_wait_1();
+    float* st = sm + b * C::STAGE;
+    // the support term onto this thread's own pieces of R
+#pragma unroll
+    for (int u = 0; u < NV; ++u) {
+      const int e = tid + 256 * u;
+      float4* d = (float4*)(st + (4 * e / RP) * SR + 4 * e % RP);
+      float4 v = *d;
+      v.x += sv[u].x; v.y += sv[u].y; v.z += sv[u].z; v.w += sv[u].w;
+      *d = v;
+    }
+    __syncthreads();
+    if (more) load_rs(t1, f, sv);
+    load_flags(t2, f);
+    if (counter && tid == 0) {
+      if ((t2 & 3) == 1) next_batch = drawn;
+      if ((t2 & 3) == 0) drawn = atomicAdd(counter, 1) + (int)gridDim.x;
+    }
+    float acc[NT][4];
+#pragma unroll
+    for (int n = 0; n < NT; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks) {
+      const float* a0 = st + (r0 + g) * SR + 16 * ks + c2;
+      uint32_t ah[4], al[4];
+      const float2 v0 = *(const float2*)a0, v1 = *(const float2*)(a0 + 8 * SR);
+      const float2 v2 = *(const float2*)(a0 + 8), v3 = *(const float2*)(a0 + 8 * SR + 8);
+      split_pair(v0.x, v0.y, ah[0], al[0]);
+      split_pair(v1.x, v1.y, ah[1], al[1]);
+      split_pair(v2.x, v2.y, ah[2], al[2]);
+      split_pair(v3.x, v3.y, ah[3], al[3]);
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+        mma_16816(acc[n], al, bh[ks][n][0], bh[ks][n][1]);
+        mma_16816(acc[n], ah, bl[ks][n][0], bl[ks][n][1]);
+        mma_16816(acc[n], ah, bh[ks][n][0], bh[ks][n][1]);
+      }
+    }
+    __syncthreads();   // every warp has read its rows of the tile: X replaces it
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+      float* o = st + (r0 + g) * SR + nw + 8 * n + c2;
+      *(float2*)o = make_float2(acc[n][0], acc[n][1]);
+      *(float2*)(o + 8 * SR) = make_float2(acc[n][2], acc[n][3]);
+    }
+    __syncthreads();
+    int64_t row;
+    const int nr = rows_of(t, row);
+#pragma unroll
+    for (int u = 0; u < NV; ++u) {
+      const int e = tid + 256 * u, i = 4 * e / RP, c = 4 * e % RP;
+      if (i >= nr) continue;
+      const float4 x4 = *(const float4*)(st + i * SR + c);
+      const float4 m4 = *(const float4*)(st + TR * SR + 4 * e);
+      const float x[4] = {x4.x, x4.y, x4.z, x4.w}, mo[4] = {m4.x, m4.y, m4.z, m4.w};
+      float eo[4] = {0.f, 0.f, 0.f, 0.f}, nv[4], ev[4];
+      if (momentum) {
+        const float4 e4 = *(const float4*)(st + TR * SR + TR * RP + 4 * e);
+        eo[0] = e4.x; eo[1] = e4.y; eo[2] = e4.z; eo[3] = e4.w;
+      }
+      bool finite = true;
+      uint32_t hw[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float uv = delta_form ? eta * x[j] : eta * (x[j] - mo[j]);
+        ev[j] = momentum ? fmaf(gamma, eo[j], uv) : uv;
+        nv[j] = mo[j] + ev[j];
+        finite = finite && isfinite(nv[j]);
+        hw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(nv[j]));
+      }
+      const int64_t o = (m0 + row + i) * RP + c;
+      *(float4*)(M + o) = make_float4(nv[0], nv[1], nv[2], nv[3]);
+      if (momentum) *(float4*)(E + o) = make_float4(ev[0], ev[1], ev[2], ev[3]);
+      *(uint2*)(Mhi + o) = make_uint2(hw[0] | (hw[1] << 16), hw[2] | (hw[3] << 16));
+      if (!finite) set_status(status, NMD_ERR_DIVERGED, (int)(m0 + row + i), 0);
+    }
+    if (!more) break;
+    __syncthreads();   // this stage is refilled by the next iteration's copies
+    t = t1;
+    t1 = t2;
+    if (counter) t2 = (t2 & 3) != 3 ? t2 + 1 : 4 * (int64_t)next_batch;
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// ---------------------------------------------------------------------------
 // Loss, support part: for every stored (i, j), with L = w_i . b_j and
 // Shat = max(0, L):
 //   a = (S - L)^2,  b = (S - Shat)^2,  mn = min(S, Shat),  mx = max(S, Shat)
@@ -1903,18 +2122,19 @@ int launch_sparse(const StepArgs& a, const PanelRow* rows, int64_t nrows, const 
   // The support term reads the same factor values as the rest of the step's
   // least-squares problem: the bf16 pieces in the bf16 mode (whose dense term
   // and Gram matrix are formed from them), the fp32 masters otherwise.
+  constexpr int kW = kSparseThreads / 32;   // warps per block
 #define NMD_SP(RPV, LPE, CPL, TT, MOP, QOP)                                                                  \
   do {                                                                                                       \
     if (nrows > 0) {                                                                                         \
       constexpr int rpw = 32 / ((RPV) / (16 / (int)sizeof(TT)) < 32 ? (RPV) / (16 / (int)sizeof(TT)) : 32);  \
-      const int64_t nb = (nrows + 8 * rpw - 1) / (8 * rpw);                                                  \
-      sparse_group_kernel<RPV, TT><<<(unsigned)nb, 256, 0, s>>>(rows, nrows, MOP, a.m0, QOP, qidx, vals, R); \
+      const int64_t nb = (nrows + kW * rpw - 1) / (kW * rpw);                                                \
+      sparse_group_kernel<RPV, TT><<<(unsigned)nb, kSparseThreads, 0, s>>>(rows, nrows, MOP, a.m0, QOP, qidx, vals, R); \
     }                                                                                                        \
     if (nwhole > 0)                                                                                          \
-      sparse_long_kernel<LPE, CPL, TT><<<(unsigned)((nwhole + 7) / 8), 256, 0, s>>>(                          \
+      sparse_long_kernel<LPE, CPL, TT><<<(unsigned)((nwhole + kW - 1) / kW), kSparseThreads, 0, s>>>(                          \
           whole, nwhole, MOP, a.m0, QOP, qidx, vals, R, nullptr, a.rp);                                      \
     if (nseg > 0) {                                                                                          \
-      sparse_long_kernel<LPE, CPL, TT><<<(unsigned)((nseg + 7) / 8), 256, 0, s>>>(                            \
+      sparse_long_kernel<LPE, CPL, TT><<<(unsigned)((nseg + kW - 1) / kW), kSparseThreads, 0, s>>>(                            \
           seg, nseg, MOP, a.m0, QOP, qidx, vals, R, seg_partials, a.rp);                                     \
       launch_reduce(multi, nmulti, partials, R, a.m0, a.rp, s);                                              \
     }                                                                                                        \
@@ -1971,22 +2191,68 @@ static void update_rp(const StepArgs& a, const float* R, const float* Rs, const 
 // per factor, three products, fp32 accumulation: mma.sync, since the SMs the
 // deferred update shares with the dense kernel have no tensor memory free),
 // in the other modes on the CUDA cores in fp32
+template <int RP>
+static bool update_tc_rp(const StepArgs& a, int64_t n0, int64_t r1, int64_t n1, const float* R, const float* Rs,
+                         const uint8_t* flags, const bf16* gsplit, float eta, float gamma, bool momentum,
+                         int* counter, int* status, cudaStream_t s) {
+  using C = UpdTc<RP>;
+  static std::atomic<int> attr[kMaxDevices];
+  // the largest shared-memory configuration, like the dense kernel's, so that
+  // an SM running an update block can take a dense CTA and vice versa
+  if (!per_device(attr, [] {
+        return cudaFuncSetAttribute(update_tc_kernel<RP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)C::SMEM) == cudaSuccess &&
+                       cudaFuncSetAttribute(update_tc_kernel<RP>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                            100) == cudaSuccess ? 1 : 0;
+      }))
+    return false;
+  const int64_t tiles = (n0 + C::TR - 1) / C::TR + (n1 + C::TR - 1) / C::TR;
+  if (tiles == 0) return true;
+  // deferred (counter): one block per SM, see the kernel; at r_pad <= 32, whose
+  // tiles are a few KB, a block per tile (connectome r = 16: 66 us as one block
+  // per SM beside a dense kernel of 41 us)
+  if (RP < 64) counter = nullptr;
+  if (counter && cudaMemsetAsync(counter, 0, sizeof(int), s) != cudaSuccess) return false;
+  const int64_t grid = counter ? std::min<int64_t>((tiles + 3) / 4, a.num_sms) : tiles;
+  const Factor& f = *a.fm;
+  update_tc_kernel<RP><<<(unsigned)grid, 256, C::SMEM, s>>>(f.master, f.hi, f.E, a.m0, n0, r1, n1, R, Rs, flags, gsplit,
+                                                          eta, gamma, momentum, a.epilogue == NMD_EPI_DELTA, counter,
+                                                          status);
+  return true;
+}
+
+bool update_takes_ranges(const StepArgs& a, const bf16* gsplit) {
+  return a.precision == NMD_BF16 && gsplit != nullptr && a.rp <= 64;
+}
+
+bool launch_update_ranges(const StepArgs& a, int64_t n0, int64_t r1, int64_t n1, const float* R, const float* Rs,
+                          const uint8_t* flags, const bf16* gsplit, float eta, float gamma, bool momentum,
+                          int* counter, int* status, cudaStream_t s) {
+  switch (a.rp) {
+    case 16: return update_tc_rp<16>(a, n0, r1, n1, R, Rs, flags, gsplit, eta, gamma, momentum, counter, status, s);
+    case 32: return update_tc_rp<32>(a, n0, r1, n1, R, Rs, flags, gsplit, eta, gamma, momentum, counter, status, s);
+    case 64: return update_tc_rp<64>(a, n0, r1, n1, R, Rs, flags, gsplit, eta, gamma, momentum, counter, status, s);
+  }
+  return false;
+}
+
 void launch_update(const StepArgs& a, const float* R, const float* Rs, const uint8_t* flags, const float* Ginv,
                    const bf16* gsplit, float eta, float gamma, bool momentum, int* status, cudaStream_t s) {
+  // r_pad = 128 in the bf16 mode: 32-row tiles where the rows fill fewer
+  // 64-row tiles than there are SMs
   const bool tc = a.precision == NMD_BF16 && gsplit != nullptr;
-  // 32-row tiles where the rows fill fewer 64-row tiles than there are SMs
   const bool small = a.M < (int64_t)a.num_sms * 64;
   switch (a.rp) {
-#define NMD_UPD(RPV)                                                                                          \
-  (!tc ? update_rp<RPV, false>(a, R, Rs, flags, Ginv, gsplit, eta, gamma, momentum, status, s)                 \
-       : (small && RPV >= 32) ? update_rp<RPV, true, (RPV >= 32 ? 32 : 64)>(a, R, Rs, flags, Ginv, gsplit, eta, \
-                                                                            gamma, momentum, status, s)        \
-                              : update_rp<RPV, true>(a, R, Rs, flags, Ginv, gsplit, eta, gamma, momentum, status, s))
-    case 16: NMD_UPD(16); break;
-    case 32: NMD_UPD(32); break;
-    case 64: NMD_UPD(64); break;
-    case 128: NMD_UPD(128); break;
-    default: update_rp<256, false>(a, R, Rs, flags, Ginv, gsplit, eta, gamma, momentum, status, s); break;
+#define NMD_UPD(...) update_rp<__VA_ARGS__>(a, R, Rs, flags, Ginv, gsplit, eta, gamma, momentum, status, s)
+    case 16: NMD_UPD(16, false); break;
+    case 32: NMD_UPD(32, false); break;
+    case 64: NMD_UPD(64, false); break;
+    case 128:
+      if (!tc) NMD_UPD(128, false);
+      else if (small) NMD_UPD(128, true, 32);
+      else NMD_UPD(128, true, 64);
+      break;
+    default: NMD_UPD(256, false); break;
 #undef NMD_UPD
   }
 }

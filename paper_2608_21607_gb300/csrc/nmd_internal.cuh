@@ -140,7 +140,7 @@ struct Workspace {
   double* loss_part = nullptr; // kLossParts x 8
   double* loss_out = nullptr;  // 8
   int* status = nullptr;       // kStatusWords
-  int* counters = nullptr;     // 64 ints; ints 0-1: skipped Delta-form chunks (u64)
+  int* counters = nullptr;     // 64 ints; 0-1: skipped Delta-form chunks (u64), 2: deferred update's tiles
   float* seg_partials = nullptr;  // max segments x rp (sparse correction of long rows)
   uint8_t* flags = nullptr;       // the panels' support-row flags, concatenated
   float* rpart = nullptr;         // kRpartRows x rp: partial R's of split-K steps
@@ -269,6 +269,14 @@ int launch_sparse(const StepArgs& a, const PanelRow* rows, int64_t nrows, const 
 void launch_update(const StepArgs& a, const float* R, const float* Rs, const uint8_t* flags,
                    const float* Ginv, const bf16* gsplit, float eta, float gamma, bool momentum, int* status,
                    cudaStream_t s);
+// The bf16 mode's update at r_pad <= 64 over the rows [0, n0) and [r1, r1 + n1)
+// of the step's M side; with a counter (device int, used by this launch
+// alone until it ends) as a deferred update beside other kernels: one block
+// per SM.  False when a CUDA call failed.
+bool update_takes_ranges(const StepArgs& a, const bf16* gsplit);
+bool launch_update_ranges(const StepArgs& a, int64_t n0, int64_t r1, int64_t n1, const float* R, const float* Rs,
+                          const uint8_t* flags, const bf16* gsplit, float eta, float gamma, bool momentum,
+                          int* counter, int* status, cudaStream_t s);
 void launch_combine(float* R, const float* Rs, const uint8_t* flags, int64_t rows, int rp, cudaStream_t s);
 // the bounded pipeline wait, run on a barrier that never completes
 void launch_wait_selftest(int* status, uint64_t limit_ns, cudaStream_t s);

@@ -39,6 +39,7 @@
 // NMD_ERR_TIMEOUT, the other roles stop at their next wait, in-flight MMAs
 // and copies are drained and TMEM is freed before the kernel returns.
 #include <cudaTypedefs.h>
+#include <limits.h>
 
 #include <algorithm>
 #include <map>
@@ -56,10 +57,9 @@ using namespace tc;
 constexpr int kEpiThreads = 256;                 // two epilogue warpgroups
 constexpr int kProducerWarp = 8, kMma1Warp = 9, kMma2Warp = 10;
 constexpr int kThreads = 352;
-// Launch bound of the panel kernel at r_pad <= 64: caps its registers at 128 a
-// thread, so that an update block (256 threads of 80) finds room in the
-// register file beside a CTA (352 x 128 + 256 x 80 = 65,536).
-constexpr int kRegThreads = 512;
+// The panel kernel's registers are capped at 112: the three of its warps on an
+// SM sub-partition then leave room (16,384 - 3 x 32 x 112 registers) for two
+// warps of 80 registers, an update block's share, and for a Gram block's.
 constexpr int BM = 128;
 constexpr uint64_t kTimeoutNs = 2000000000ull;
 
@@ -123,7 +123,10 @@ struct Cfg {
   static constexpr size_t OFF_W = (size_t)NSTAGE * STAGE_BYTES;
   static constexpr int W_PANEL_BYTES = BM * ROWB;     // one swizzle panel of a W tile
   static constexpr size_t OFF_STG = OFF_W + (size_t)NWB * W_BYTES;
-  static constexpr size_t OFF_BARS = OFF_STG + STG_BYTES;
+  // loss pass: each epilogue thread's window of column indices (16, at a stride of 17)
+  static constexpr size_t OFF_WIN = OFF_STG;
+  static constexpr int WIN_BYTES = LOSS ? kEpiThreads * 17 * 4 : 0;
+  static constexpr size_t OFF_BARS = OFF_STG + STG_BYTES + WIN_BYTES;
   static constexpr int COL_L = 0;                     // NB x BN columns
   static constexpr int COL_R = NB * BN;               // NRB x RCOLS columns
   static constexpr int COL_W = COL_R + NRB * RCOLS;   // NWB x WCOLS columns
@@ -379,7 +382,7 @@ __device__ __noinline__ void store_r_tile(uint32_t tmem_r, uint32_t b_rempty, fl
 // products of the chunks that the range-search mask clears.  Separate
 // instantiations, so that the kernel without them carries none of the checks.
 template <int RP, int EPI, bool SPLIT, int MODE, int SKIPM>
-__global__ void __launch_bounds__(MODE == 0 ? kRegThreads : kThreads, 1)
+__global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 104 : 112) : 168)
     panel_tc_kernel(const __grid_constant__ CUtensorMap tq_hi, const __grid_constant__ CUtensorMap tq_lo,
                     const __grid_constant__ CUtensorMap tq_lo2, const __grid_constant__ CUtensorMap tw,
                     const TcParams p) {
@@ -735,8 +738,10 @@ __global__ void __launch_bounds__(MODE == 0 ? kRegThreads : kThreads, 1)
     bool ok = true;
     // loss pass: this thread's row of S, walked alongside the column chunks so
     // that support entries are left to the support pass (no cancellation)
-    int64_t se = 0, send = 0;
-    int64_t snext = INT64_MAX;
+    constexpr int kWin = 16;
+    int64_t se = 0, send = 0;              // the row's entries from the window's first to its last
+    int wpos = 0, wcnt = 0;                // position in the window, entries in it
+    int* win = (int*)(smem + C::OFF_WIN) + et * (kWin + 1);
 
     // load the W tile `tile` into W buffer wb: warpgroup g takes 8-word groups g, g+2, ...
     auto load_w = [&](int64_t tile, int wb) {
@@ -799,66 +804,79 @@ __global__ void __launch_bounds__(MODE == 0 ? kRegThreads : kThreads, 1)
       if (lane == 0) mbar_arrive(b_wfull + 8 * wb);
     };
 
-    // Loss pass: this row's entries in columns [c0, c0 + BN) as bits, the row's
-    // position moved past them.  A row's first entries of the chunk are read
-    // by its own thread; what is left of a longer one (a hub of the graph has
-    // an entry in every column, 128 dependent loads per chunk) by the whole warp,
-    // 32 entries at a time.  The other warpgroup's chunks are passed over by
-    // a doubling search.  Called by converged warps.
+    // Loss pass: this row's entries in columns [c0, c0 + BN) as bits, c0
+    // ascending within a tile.  The row's next entries sit in a window of
+    // kWin column indices in shared memory (a dependent global load per entry
+    // held the epilogue up for most of the pass: 8.1 ms at 139,255 nodes and 2.8M
+    // entries), refilled by the row's own thread, its loads in flight
+    // together.  A row that needs more than one refill within a chunk (a hub
+    // of the graph has an entry in every column) is read on by the whole
+    // warp, 256 entries at a time.  Called by converged warps.
+    auto refill = [&](int64_t from) {   // this thread's window: entries [from, from + kWin) of its row
+      se = from;
+      wpos = 0;
+      wcnt = (int)(send - from < kWin ? send - from : kWin);
+      int col[kWin];
+#pragma unroll
+      for (int i = 0; i < kWin; ++i) col[i] = i < wcnt ? p.cidx[from + i] : 0;
+#pragma unroll
+      for (int i = 0; i < kWin; ++i) win[i] = col[i];
+    };
     auto support_mask = [&](int64_t c0, uint32_t(&msk)[BN / 32]) {
-      constexpr int W = BN / 32, kOwn = 8;
+      constexpr int W = BN / 32;
       const int64_t cend = c0 + BN;
 #pragma unroll
       for (int w = 0; w < W; ++w) msk[w] = 0u;
-      if (snext < c0) {   // first entry at or past column c0
-        int64_t step = 1, lo = se;   // cidx[lo] < c0
-        while (lo + step < send && p.cidx[lo + step] < c0) {
-          lo += step;
-          step *= 2;
-        }
-        int64_t hi = lo + step < send ? lo + step : send;
-        while (hi - lo > 1) {
-          const int64_t mid = lo + (hi - lo) / 2;
-          if (p.cidx[mid] < c0) lo = mid;
-          else hi = mid;
-        }
-        se = hi;
-        snext = se < send ? p.cidx[se] : INT64_MAX;
-      }
-      for (int n = 0; n < kOwn && snext < cend; ++n) {
-        const int b = (int)(snext - c0);
-#pragma unroll
-        for (int w = 0; w < W; ++w)
-          if (w == (b >> 5)) msk[w] |= 1u << (b & 31);
-        ++se;
-        snext = se < send ? p.cidx[se] : INT64_MAX;
-      }
-      uint32_t more = __ballot_sync(0xffffffffu, snext < cend);
-      while (more) {
-        const int src = __ffs(more) - 1;
-        more &= more - 1;
-        int64_t q = __shfl_sync(0xffffffffu, se, src);
-        const int64_t e = __shfl_sync(0xffffffffu, send, src);
-        uint32_t m[W];
-#pragma unroll
-        for (int w = 0; w < W; ++w) m[w] = 0u;
-        int n;
-        do {
-          const int64_t col = q + lane < e ? (int64_t)p.cidx[q + lane] : INT64_MAX;
-          const bool in = col < cend;
-          const int b = in ? (int)(col - c0) : 0;
+      for (int pass = 0;; ++pass) {
+        for (; wpos < wcnt; ++wpos) {
+          const int64_t col = win[wpos];
+          if (col >= cend) break;
+          const int b = (int)(col - c0);
 #pragma unroll
           for (int w = 0; w < W; ++w)
-            m[w] |= __reduce_or_sync(0xffffffffu, in && (b >> 5) == w ? 1u << (b & 31) : 0u);
-          n = __popc(__ballot_sync(0xffffffffu, in));
-          q += n;
-        } while (n == 32);
-        if (lane == src) {
-#pragma unroll
-          for (int w = 0; w < W; ++w) msk[w] |= m[w];
-          se = q;
-          snext = se < send ? p.cidx[se] : INT64_MAX;
+            if (b >= 0 && w == (b >> 5)) msk[w] |= 1u << (b & 31);
         }
+        const bool out = wpos == wcnt && se + wcnt < send;   // the window is used up, the row is not
+        uint32_t more = __ballot_sync(0xffffffffu, out);
+        if (more == 0u) break;
+        if (pass == 0 || __popc(more) > 4) {
+          if (out) refill(se + wcnt);
+          continue;
+        }
+        while (more) {
+          const int src = __ffs(more) - 1;
+          more &= more - 1;
+          int64_t q = __shfl_sync(0xffffffffu, se + wcnt, src);
+          const int64_t e = __shfl_sync(0xffffffffu, send, src);
+          uint32_t m[W];
+#pragma unroll
+          for (int w = 0; w < W; ++w) m[w] = 0u;
+          int n;
+          do {
+            int col[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) col[k] = q + lane + 32 * k < e ? p.cidx[q + lane + 32 * k] : INT_MAX;
+            n = 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const bool in = col[k] < cend && col[k] != INT_MAX;
+              n += __popc(__ballot_sync(0xffffffffu, in));
+              const int64_t b = (int64_t)col[k] - c0;
+              if (__any_sync(0xffffffffu, in && b >= 0))
+#pragma unroll
+                for (int w = 0; w < W; ++w)
+                  m[w] |= __reduce_or_sync(0xffffffffu, in && b >= 0 && (int)(b >> 5) == w ? 1u << ((int)b & 31) : 0u);
+            }
+            q += n;
+          } while (n == 256);
+          if (lane == src) {
+#pragma unroll
+            for (int w = 0; w < W; ++w) msk[w] |= m[w];
+            refill(q);
+          }
+          __syncwarp();
+        }
+        break;   // those rows' windows now start past the chunk, or their rows end
       }
     };
 
@@ -889,9 +907,8 @@ __global__ void __launch_bounds__(MODE == 0 ? kRegThreads : kThreads, 1)
       const ChunkMask cm = chunk_mask<RANGE>(p, t, kc0, nchunks, &clast, &nlive);
       if (SUMS) {
         const int64_t li = (int64_t)t * BM + row;
-        se = li < p.M ? p.rowptr[li] : 0;
         send = li < p.M ? p.rowptr[li + 1] : 0;
-        snext = se < send ? p.cidx[se] : INT64_MAX;
+        refill(li < p.M ? p.rowptr[li] : 0);
       }
       for (int ci = 0; ci < (int)nchunks; ++ci) {
         if (RANGE && !cm.live(ci)) continue;
