@@ -291,7 +291,7 @@ void layout(Carver& c, int64_t m, int64_t n, int64_t nnz, int rp, int64_t npanel
   w->R2 = c.take<float>(std::max(m, n) * rp);
   w->Rs = c.take<float>(std::max(m, n) * rp);
   w->Rs2 = c.take<float>(std::max(m, n) * rp);
-  w->gram_part = c.take<float>((size_t)kGramParts * rp * rp);
+  w->gram_part = c.take<float>((size_t)(kGramParts + 8) * rp * rp);
   w->G = c.take<float>((size_t)rp * rp);
   w->Ginv = c.take<float>((size_t)rp * rp);
   w->G2 = c.take<float>((size_t)rp * rp);
@@ -771,13 +771,15 @@ nmd_status run_step_roles(nmd_handle* h, const Roles& ro, int kind, bool do_upda
   CK(h, cudaStreamWaitEvent(h->side2, h->ev_fork, 0));
   if (need_gram) {
     TimedScope ts(h, NMD_K_GRAM, h->side);
-    if (!gram_first) {
-      launch_gram_parts(ro.fq, rounded, ro.q0, ro.K, h->rp, h->ws.gram_part, nparts, chunk, h->side);
+    if (launch_gram_inv(ro.fq, rounded, ro.q0, ro.K, h->r, h->rp, h->ws.gram_part,
+                        h->ws.gram_part + (size_t)kGramParts * h->rp * h->rp, nparts, chunk, (float)h->opt.ridge, G,
+                        Ginv, gsplit_of(h, Ginv), h->ws.counters + 8, h->ws.status, h->side)) {
       h->launches++;
+    } else {
+      launch_gram_reduce(h->ws.gram_part, nparts, h->r, h->rp, (float)h->opt.ridge, G, h->side);
+      launch_chol_inv(G, h->r, h->rp, Ginv, gsplit_of(h, Ginv), h->ws.status, h->side);
+      h->launches += 2;
     }
-    launch_gram_reduce(h->ws.gram_part, nparts, h->r, h->rp, (float)h->opt.ridge, G, h->side);
-    launch_chol_inv(G, h->r, h->rp, Ginv, gsplit_of(h, Ginv), h->ws.status, h->side);
-    h->launches += 2;
     if (tc_update(h)) {   // the pieces of G^{-1} for the tensor-core update
       Factor gi = *gi_of(h, Ginv);
       launch_pack(Ginv, false, h->rp, h->rp, h->rp, gi, h->side);

@@ -232,34 +232,32 @@ __global__ void __launch_bounds__(256) small_gemm_kernel(const float* __restrict
 //     (two buffers) and every row below subtracts sum_k l_ik Y[k, :].  One
 //     barrier per panel.
 //  3. G^{-1} = Y^T D^{-1} Y from shared memory.
-// entry (k, n) of G^{-1} as hi + lo bf16 pieces at row n, column k of the
-// transposed split (hi rows first, then lo rows)
-template <int RP>
-__device__ __forceinline__ void store_split(bf16* gsplit, int n, int k, float v) {
-  constexpr int SB = split_stride(RP);
-  const bf16 hi = __float2bfloat16_rn(v);
-  gsplit[n * SB + k] = hi;
-  gsplit[RP * SB + n * SB + k] = __float2bfloat16_rn(v - __bfloat162float(hi));
+// two entries of G^{-1} as hi + lo bf16 pieces, packed in pairs
+__device__ __forceinline__ void split2(float x0, float x1, uint32_t& hi, uint32_t& lo) {
+  const bf16 h0 = __float2bfloat16_rn(x0), h1 = __float2bfloat16_rn(x1);
+  const bf16 l0 = __float2bfloat16_rn(x0 - __bfloat162float(h0)), l1 = __float2bfloat16_rn(x1 - __bfloat162float(h1));
+  hi = __bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+  lo = __bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
 }
 
+// (run by the first 4 RP threads of a block; `bad`: shared; G is read past L1,
+// it was written by other blocks of the same kernel)
 template <int RP>
-__global__ void __launch_bounds__(RP * 4) ldlt_inv_reg_kernel(const float* __restrict__ G, int r,
-                                                              float* __restrict__ Ginv, bf16* __restrict__ gsplit,
-                                                              int* __restrict__ status) {
+__device__ void ldlt_inv_reg(const float* G, int r, float* __restrict__ Ginv, bf16* __restrict__ gsplit,
+                             int* __restrict__ status, float* smr, volatile int& bad) {
   constexpr int CPT = RP / 4, PB = CPT < 8 ? CPT : 8, LD = RP + 1;
-  extern __shared__ __align__(16) float smr[];
+  auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(RP * 4) : "memory"); };
   float* invd = smr;                 // RP: 1 / d_k
   float* diag0 = invd + RP;          // RP: the diagonal of G
   float* DB = diag0 + RP;            // PB x PB: the diagonal block being factored (64 floats)
   float* Pn = DB + 64;               // RP x PB: the panel's columns / 2 x PB x RP: rows of Y
   float* F = Pn + 2 * PB * RP;       // RP x LD: the factor, then Y
-  __shared__ int bad;
   const int i = threadIdx.x / 4, s = threadIdx.x % 4, c0 = s * CPT, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) bad = 0;
   float a[CPT];
 #pragma unroll
   for (int j = 0; j < CPT; j += 4) {
-    const float4 v = *(const float4*)(G + (size_t)i * RP + c0 + j);
+    const float4 v = __ldcg((const float4*)(G + (size_t)i * RP + c0 + j));
     a[j] = v.x; a[j + 1] = v.y; a[j + 2] = v.z; a[j + 3] = v.w;
   }
 #pragma unroll
@@ -268,7 +266,7 @@ __global__ void __launch_bounds__(RP * 4) ldlt_inv_reg_kernel(const float* __res
       if (i >= r) a[j] = 1.f;
       diag0[i] = a[j];
     }
-  __syncthreads();
+  sync();
   const float tol = 4.0f * (float)r * FLT_EPSILON;
   // 1. G = L D L^T, a[] keeping a_ij = l_ij d_j (j < i) and d_i (j == i)
 #pragma unroll
@@ -310,7 +308,7 @@ __global__ void __launch_bounds__(RP * 4) ldlt_inv_reg_kernel(const float* __res
           DB[qo * PB + k] = blk[k];
         }
     }
-    __syncthreads();
+    sync();
     if (bad) {   // uniform: every thread reads the flag after the barrier
 #pragma unroll
       for (int j = 0; j < CPT; ++j) Ginv[(size_t)i * RP + c0 + j] = 0.f;
@@ -329,7 +327,7 @@ __global__ void __launch_bounds__(RP * 4) ldlt_inv_reg_kernel(const float* __res
       for (int k = 0; k < PB; k += 4)
         *(float4*)(Pn + i * PB + k) = make_float4(a[jp + k], a[jp + k + 1], a[jp + k + 2], a[jp + k + 3]);
     }
-    __syncthreads();
+    sync();
     if (i >= kb + PB) {
       float u[PB];
 #pragma unroll
@@ -355,7 +353,7 @@ __global__ void __launch_bounds__(RP * 4) ldlt_inv_reg_kernel(const float* __res
   }
 #pragma unroll
   for (int j = 0; j < CPT; ++j) F[i * LD + c0 + j] = a[j];
-  __syncthreads();
+  sync();
   // 2. Y = L^{-1} (a[] now holds row i of Y), l_ik = a_ik / d_k
 #pragma unroll
   for (int j = 0; j < CPT; ++j) a[j] = c0 + j == i ? 1.f : 0.f;
@@ -379,7 +377,7 @@ __global__ void __launch_bounds__(RP * 4) ldlt_inv_reg_kernel(const float* __res
         for (int jj = 0; jj < CPT; jj += 4)
           *(float4*)(YP + rl * RP + c0 + jj) = make_float4(a[jj], a[jj + 1], a[jj + 2], a[jj + 3]);
     }
-    __syncthreads();
+    sync();
     if (i >= kb + PB) {
       float l[PB];
 #pragma unroll
@@ -397,10 +395,10 @@ __global__ void __launch_bounds__(RP * 4) ldlt_inv_reg_kernel(const float* __res
       }
     }
   }
-  __syncthreads();   // every read of the factor is done
+  sync();   // every read of the factor is done
 #pragma unroll
   for (int j = 0; j < CPT; ++j) F[i * LD + c0 + j] = a[j];
-  __syncthreads();
+  sync();
   // 3. G^{-1}[i][j] = sum over k of Y[k][i] Y[k][j] / d_k (Y[k][j] = 0 for j > k)
 #pragma unroll
   for (int j = 0; j < CPT; ++j) a[j] = 0.f;
@@ -414,14 +412,22 @@ __global__ void __launch_bounds__(RP * 4) ldlt_inv_reg_kernel(const float* __res
 #pragma unroll
   for (int j = 0; j < CPT; j += 4)
     *(float4*)(Ginv + (size_t)i * RP + c0 + j) = make_float4(a[j], a[j + 1], a[j + 2], a[j + 3]);
-  if (gsplit)
+  if (gsplit) {   // transposed through shared memory: row n of the pieces is column n of G^{-1}
+    sync();       // every read of Y is done
 #pragma unroll
-    for (int j = 0; j < CPT; ++j) store_split<RP>(gsplit, c0 + j, i, a[j]);
-}
-
-inline size_t ldlt_reg_smem_bytes(int rp) {
-  const size_t pb = rp / 4 < 8 ? rp / 4 : 8;
-  return ((size_t)2 * rp + 64 + 2 * pb * rp + (size_t)rp * (rp + 1)) * sizeof(float);
+    for (int j = 0; j < CPT; ++j) F[i * LD + c0 + j] = a[j];
+    sync();
+    uint32_t hw[CPT / 2], lw[CPT / 2];
+#pragma unroll
+    for (int j = 0; j < CPT; j += 2) split2(F[(c0 + j) * LD + i], F[(c0 + j + 1) * LD + i], hw[j / 2], lw[j / 2]);
+    uint32_t* hi = reinterpret_cast<uint32_t*>(gsplit + i * split_stride(RP) + c0);
+    uint32_t* lo = reinterpret_cast<uint32_t*>(gsplit + (RP + i) * split_stride(RP) + c0);
+#pragma unroll
+    for (int j = 0; j < CPT / 2; ++j) {
+      hi[j] = hw[j];
+      lo[j] = lw[j];
+    }
+  }
 }
 
 // Tile-blocked form of the same factorisation for r_pad in {64, 128, 256}:
@@ -453,7 +459,11 @@ struct TileChol {
   static constexpr int NTILE = NT * (NT + 1) / 2;
   static constexpr int NTHR = RP * 4 > 512 ? 512 : RP * 4;
   static constexpr int PBUF = TB * RP;   // the transposed panel (32 x RP), or the T_IJ of one tile row
-  static constexpr size_t SMEM = ((size_t)NTILE * TSZ + PBUF + 3 * RP) * sizeof(float);
+  // r_pad <= 128: G^{-1} is assembled in shared memory and leaves in whole rows
+  static constexpr bool STAGED = RP <= 128;
+  static constexpr int LDO = RP + 1;
+  static constexpr size_t SMEM =
+      ((size_t)NTILE * TSZ + PBUF + 3 * RP + (STAGED ? (size_t)RP * LDO : 0)) * sizeof(float);
   static_assert(RP % TB == 0 && NT >= 2, "tile form for r_pad >= 64");
 };
 
@@ -466,39 +476,43 @@ __device__ __forceinline__ void tile_of(int q, int& I, int& J) {
   J = q - ((I * (I + 1)) >> 1);
 }
 
-// (registers capped at 64: beside a dense CTA of r_pad = 64 there are 20,480 left
-// on an SM, which 256 threads of 128 did not fit into, so that the inverse waited
-// for an SM without a dense CTA: 105 -> 78 us for the Gram chain beside it; at
-// r_pad = 256 512 threads of 64 find room beside the support term's blocks)
-template <int RP>
-__global__ void __launch_bounds__(1024, 1) ldlt_inv_tile_kernel(const float* __restrict__ G, int r,
-                                                                          float* __restrict__ Ginv,
-                                                                          bf16* __restrict__ gsplit,
-                                                                          int* __restrict__ status) {
+// (G is read past L1: at r_pad = 64 it was written by the same kernel)
+template <int RP, int NTHR>
+__device__ void ldlt_inv_tile(const float* G, int r, float* __restrict__ Ginv, bf16* __restrict__ gsplit,
+                              int* __restrict__ status, float* smt, volatile int& bad) {
   using C = TileChol<RP>;
-  constexpr int TB = C::TB, NT = C::NT, LDT = C::LDT, TSZ = C::TSZ, NTHR = C::NTHR;
-  extern __shared__ __align__(16) float smt[];
+  constexpr int TB = C::TB, NT = C::NT, LDT = C::LDT, TSZ = C::TSZ;
   float* A = smt;                        // NTILE tiles: the matrix, then L and Y
   float* P = A + C::NTILE * TSZ;         // PBUF
   float* dv = P + C::PBUF;               // RP: d_k
   float* invd = dv + RP;                 // RP: 1 / d_k
   float* diag0 = invd + RP;              // RP: the diagonal of G
-  __shared__ int bad;
+  float* out = diag0 + RP;               // STAGED: RP x LDO, G^{-1}
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) bad = 0;
-  for (int t = tid; t < C::NTILE * TB * TB; t += NTHR) {
+  // (G is zero past r; the pads of its diagonal are set to one)
+#pragma unroll 4
+  for (int t = tid; t < C::NTILE * TB * TB / 4; t += NTHR) {
     int I, J;
-    tile_of(t / (TB * TB), I, J);
-    const int e = t % (TB * TB), ii = e / TB, jj = e % TB, i = I * TB + ii, j = J * TB + jj;
-    const float g = (i < r && j < r) ? G[(size_t)i * RP + j] : (i == j ? 1.f : 0.f);
-    A[(t / (TB * TB)) * TSZ + ii * LDT + jj] = g;
-    if (i == j) diag0[i] = g;
-  }
-  for (int e = tid; e < RP * RP; e += NTHR)
-    if (e / RP >= r || e % RP >= r) {
-      Ginv[e] = 0.f;
-      if (gsplit) store_split<RP>(gsplit, e % RP, e / RP, 0.f);
+    tile_of(t / (TB * TB / 4), I, J);
+    const int e = t % (TB * TB / 4), ii = e / (TB / 4), jj = 4 * (e % (TB / 4)), i = I * TB + ii, j = J * TB + jj;
+    const float4 g4 = __ldcg((const float4*)(G + (size_t)i * RP + j));
+    float g[4] = {g4.x, g4.y, g4.z, g4.w};
+    float* at = A + (t / (TB * TB / 4)) * TSZ + ii * LDT + jj;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (i == j + q) {
+        if (i >= r) g[q] = 1.f;
+        diag0[i] = g[q];
+      }
+      at[q] = g[q];
     }
+  }
+  if (C::STAGED)
+    for (int e = tid; e < RP * C::LDO; e += NTHR) out[e] = 0.f;
+  else
+    for (int e = tid; e < RP * RP; e += NTHR)
+      if (e / RP >= r || e % RP >= r) Ginv[e] = 0.f;
   __syncthreads();
   const float tol = 4.0f * (float)r * FLT_EPSILON;
 
@@ -509,16 +523,14 @@ __global__ void __launch_bounds__(1024, 1) ldlt_inv_tile_kernel(const float* __r
       float a[TB];
 #pragma unroll
       for (int j = 0; j < TB; ++j) a[j] = T[lane * LDT + j];
-      int badk = -1;
+      float dk = 0.f, ik = 0.f;   // this lane's d and 1 / d
 #pragma unroll
       for (int k = 0; k < TB; ++k) {
         const float d = __shfl_sync(0xffffffffu, a[k], k);
         const float inv = 1.0f / d;
-        const int kk = J * TB + k;
-        if (badk < 0 && kk < r && (!(d > tol * diag0[kk]) || !isfinite(d))) badk = kk;   // warp-uniform
         if (lane == k) {
-          dv[kk] = d;
-          invd[kk] = inv;
+          dk = d;
+          ik = inv;
         }
         const float aik = a[k];
         const float l = aik * inv;
@@ -526,6 +538,13 @@ __global__ void __launch_bounds__(1024, 1) ldlt_inv_tile_kernel(const float* __r
 #pragma unroll
         for (int j = k + 1; j < TB; ++j) a[j] = fmaf(-aik, __shfl_sync(0xffffffffu, l, j), a[j]);
       }
+      // the first bad pivot (those after it were formed from it)
+      const int kk = J * TB + lane;
+      const uint32_t wrong =
+          __ballot_sync(0xffffffffu, kk < r && (!(dk > tol * diag0[kk]) || !isfinite(dk)));
+      const int badk = wrong ? J * TB + __ffs(wrong) - 1 : -1;
+      dv[kk] = dk;
+      invd[kk] = ik;
       // the unit lower factor of the tile, then its inverse Yt in registers
 #pragma unroll
       for (int j = 0; j < TB; ++j)
@@ -682,14 +701,177 @@ __global__ void __launch_bounds__(1024, 1) ldlt_inv_tile_kernel(const float* __r
       for (int v = 0; v < 4; ++v) {
         const int ga = a0 + u, gb = b0 + v;
         if (ga < r && gb < r && (a0 != b0 || v <= u)) {
-          Ginv[(size_t)ga * RP + gb] = acc[u][v];
-          Ginv[(size_t)gb * RP + ga] = acc[u][v];
-          if (gsplit) {
-            store_split<RP>(gsplit, gb, ga, acc[u][v]);
-            store_split<RP>(gsplit, ga, gb, acc[u][v]);
+          if (C::STAGED) {
+            out[ga * C::LDO + gb] = acc[u][v];
+            out[gb * C::LDO + ga] = acc[u][v];
+          } else {
+            Ginv[(size_t)ga * RP + gb] = acc[u][v];
+            Ginv[(size_t)gb * RP + ga] = acc[u][v];
           }
         }
       }
+  }
+  if (C::STAGED) {   // G^{-1} (symmetric) and its pieces, row by row
+    __syncthreads();
+    for (int e = tid; e < RP * RP / 4; e += NTHR) {
+      const int i = 4 * e / RP, c = 4 * e % RP;
+      const float* o = out + i * C::LDO + c;
+      *(float4*)(Ginv + (size_t)i * RP + c) = make_float4(o[0], o[1], o[2], o[3]);
+      if (gsplit) {
+        uint2 h, l;
+        split2(o[0], o[1], h.x, l.x);
+        split2(o[2], o[3], h.y, l.y);
+        *(uint2*)(gsplit + i * split_stride(RP) + c) = h;
+        *(uint2*)(gsplit + (RP + i) * split_stride(RP) + c) = l;
+      }
+    }
+  }
+}
+
+// (512 threads of 64 registers: room beside the support term's blocks)
+template <int RP>
+__global__ void __launch_bounds__(1024, 1) ldlt_inv_tile_kernel(const float* __restrict__ G, int r,
+                                                              float* __restrict__ Ginv, bf16* __restrict__ gsplit,
+                                                              int* __restrict__ status) {
+  extern __shared__ __align__(16) float smt[];
+  __shared__ int bad;
+  ldlt_inv_tile<RP, TileChol<RP>::NTHR>(G, r, Ginv, gsplit, status, smt, bad);
+}
+
+// ---------------------------------------------------------------------------
+// r_pad <= 64: the whole Gram chain in one launch -- the partials (block p: rows
+// [p chunk, (p + 1) chunk)), their sum, the ridge and G^{-1}.  What bounds it is
+// latency: as three kernels the chain took 25 us at r_pad = 16 and 60 us at
+// r_pad = 64 beside the dense kernel, each launch waiting for SM room, and set
+// the pace of small steps (identity of 4,096, r = 3: 45 us a step).  Here the
+// block that finishes a class of partials last (p mod 8; the partials past the
+// last multiple of 8 belong to class 0) adds them, and the block that finishes
+// the classes last adds the eight sums in a fixed tree, writes G and
+// inverts it: the same sums in the same order as gram_reduce_kernel.
+// ctr: 9 ints, zero between launches; only one launch at a time uses them.
+// ---------------------------------------------------------------------------
+template <int RP>
+struct GramInv {
+  static constexpr int W = RP / 16;   // outputs per thread: W x W
+  static constexpr size_t INV = RP == 64 ? TileChol<64>::SMEM
+                                         : ((size_t)2 * RP + 64 + 2 * (RP / 4 < 8 ? RP / 4 : 8) * RP +
+                                            (size_t)RP * (RP + 1)) * sizeof(float);
+  static constexpr size_t STAGE = 32 * (RP + 1) * sizeof(float);
+  static constexpr size_t SMEM = INV > STAGE ? INV : STAGE;
+};
+
+template <int RP, typename T>
+__global__ void __launch_bounds__(256, 4) gram_inv_kernel(const T* __restrict__ Q, int64_t q0, int64_t K,
+                                                          int64_t chunk, int nparts, int r, float ridge,
+                                                          float* parts, float* sums, float* G,
+                                                          float* __restrict__ Ginv, bf16* __restrict__ gsplit,
+                                                          int* ctr, int* __restrict__ status) {
+  using C = GramInv<RP>;
+  constexpr int W = C::W, LD = RP + 1;
+  extern __shared__ __align__(16) float smg[];
+  __shared__ int flag, bad;
+  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16, p = blockIdx.x;
+  {
+    const int64_t k0 = (int64_t)p * chunk, k1 = min(K, k0 + chunk);
+    float acc[W][W] = {};
+    for (int64_t kb = k0; kb < k1; kb += 32) {
+#pragma unroll
+      for (int u = 0; u < 32 * RP / 256; ++u) {
+        const int e = tid + 256 * u, rr = e / RP, cc = e % RP;
+        smg[rr * LD + cc] = kb + rr < k1 ? to_f(Q[(q0 + kb + rr) * RP + cc]) : 0.f;
+      }
+      __syncthreads();
+#pragma unroll 4
+      for (int rr = 0; rr < 32; ++rr) {
+        float a[W], b[W];
+#pragma unroll
+        for (int i = 0; i < W; ++i) a[i] = smg[rr * LD + ty * W + i];
+#pragma unroll
+        for (int j = 0; j < W; ++j) b[j] = smg[rr * LD + tx * W + j];
+#pragma unroll
+        for (int i = 0; i < W; ++i)
+#pragma unroll
+          for (int j = 0; j < W; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+      }
+      __syncthreads();
+    }
+    float* o = parts + (size_t)p * RP * RP;
+#pragma unroll
+    for (int i = 0; i < W; ++i)
+#pragma unroll
+      for (int j = 0; j < W; ++j) __stcg(o + (ty * W + i) * RP + tx * W + j, acc[i][j]);
+  }
+  // the last block of this partial's class adds the class
+  const int floor8 = nparts / 8 * 8, nclass = floor8 ? 8 : 1;
+  const int q = p < floor8 ? p % 8 : 0;
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) flag = atomicAdd(ctr + q, 1) == floor8 / 8 + (q == 0 ? nparts - floor8 : 0) - 1;
+  __syncthreads();
+  if (!flag) return;
+  __threadfence();
+  // (16 bytes a load, a class's eight members in flight together; a member that
+  // is not there adds zero)
+  for (int e = 4 * tid; e < RP * RP; e += 1024) {
+    float4 x[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m)
+      x[m] = q + 8 * m < floor8 ? __ldcg((const float4*)(parts + (size_t)(q + 8 * m) * RP * RP + e))
+                                : make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      v.x += x[m].x; v.y += x[m].y; v.z += x[m].z; v.w += x[m].w;
+    }
+    if (q == 0)
+      for (int t = floor8; t < nparts; ++t) {
+        const float4 w = __ldcg((const float4*)(parts + (size_t)t * RP * RP + e));
+        v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+      }
+    __stcg((float4*)(sums + (size_t)q * RP * RP + e), v);
+  }
+  // the last class adds the classes, writes G to both triangles from the
+  // lower one (rows and columns past r are zero) and inverts it
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) flag = atomicAdd(ctr + 8, 1) == nclass - 1;
+  __syncthreads();
+  if (!flag) return;
+  __threadfence();
+  if (tid < 9) ctr[tid] = 0;
+  for (int e = 4 * tid; e < RP * RP; e += 1024) {
+    const int i = e / RP, j0 = e % RP;
+    if (j0 > i) continue;
+    float4 a[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      a[c] = c < nclass ? __ldcg((const float4*)(sums + (size_t)c * RP * RP + e)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    auto tree = [](float x0, float x1, float x2, float x3, float x4, float x5, float x6, float x7) {
+      return ((x0 + x1) + (x2 + x3)) + ((x4 + x5) + (x6 + x7));
+    };
+    const float t[4] = {tree(a[0].x, a[1].x, a[2].x, a[3].x, a[4].x, a[5].x, a[6].x, a[7].x),
+                        tree(a[0].y, a[1].y, a[2].y, a[3].y, a[4].y, a[5].y, a[6].y, a[7].y),
+                        tree(a[0].z, a[1].z, a[2].z, a[3].z, a[4].z, a[5].z, a[6].z, a[7].z),
+                        tree(a[0].w, a[1].w, a[2].w, a[3].w, a[4].w, a[5].w, a[6].w, a[7].w)};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int j = j0 + k;
+      if (j > i) continue;
+      float sum = 0.f;
+      if (i < r) {
+        sum = t[k];
+        if (i == j) sum += ridge;
+      }
+      __stcg(G + (size_t)i * RP + j, sum);
+      __stcg(G + (size_t)j * RP + i, sum);
+    }
+  }
+  __threadfence_block();
+  __syncthreads();
+  if constexpr (RP == 64) {
+    ldlt_inv_tile<64, TileChol<64>::NTHR>(G, r, Ginv, gsplit, status, smg, bad);
+  } else {
+    if (tid < 4 * RP) ldlt_inv_reg<RP>(G, r, Ginv, gsplit, status, smg, bad);
   }
 }
 
@@ -1836,30 +2018,50 @@ void launch_small_gemm(const float* A, int64_t lda, const float* B, int64_t ldb,
   small_gemm_kernel<<<grid, 256, 0, s>>>(A, lda, B, ldb, C, ldc, M, N, K);
 }
 
-void launch_chol_inv(const float* G, int r, int rp, float* Ginv, bf16* gsplit, int* status, cudaStream_t s) {
+template <int RP>
+static bool gram_inv_rp(const Factor* fq, bool rounded, int64_t q0, int64_t K, int r, float* parts, float* sums,
+                        int nparts, int64_t chunk, float ridge, float* G, float* Ginv, bf16* gsplit, int* ctr,
+                        int* status, cudaStream_t s) {
+  constexpr size_t smem = GramInv<RP>::SMEM;
+  if (rounded)
+    gram_inv_kernel<RP, bf16><<<(unsigned)nparts, 256, smem, s>>>(fq->hi, q0, K, chunk, nparts, r, ridge, parts, sums,
+                                                                  G, Ginv, gsplit, ctr, status);
+  else
+    gram_inv_kernel<RP, float><<<(unsigned)nparts, 256, smem, s>>>(fq->master, q0, K, chunk, nparts, r, ridge, parts,
+                                                                   sums, G, Ginv, gsplit, ctr, status);
+  return true;
+}
+
+bool launch_gram_inv(const Factor* fq, bool rounded, int64_t q0, int64_t K, int r, int rp, float* parts, float* sums,
+                     int nparts, int64_t chunk, float ridge, float* G, float* Ginv, bf16* gsplit, int* ctr,
+                     int* status, cudaStream_t s) {
+  static_assert(GramInv<64>::SMEM <= 48 * 1024, "shared memory without an attribute");
+#define NMD_GI(RPV) \
+  gram_inv_rp<RPV>(fq, rounded, q0, K, r, parts, sums, nparts, chunk, ridge, G, Ginv, gsplit, ctr, status, s)
   switch (rp) {
-    case 16: ldlt_inv_reg_kernel<16><<<1, 64, ldlt_reg_smem_bytes(16), s>>>(G, r, Ginv, gsplit, status); break;
-    case 32: ldlt_inv_reg_kernel<32><<<1, 128, ldlt_reg_smem_bytes(32), s>>>(G, r, Ginv, gsplit, status); break;
-    case 64:
-      ldlt_inv_tile_kernel<64><<<1, TileChol<64>::NTHR, TileChol<64>::SMEM, s>>>(G, r, Ginv, gsplit, status);
-      break;
-    case 128: {
-      static std::atomic<int> attr[kMaxDevices];
-      per_device(attr, [] {
-        return cudaFuncSetAttribute(ldlt_inv_tile_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)TileChol<128>::SMEM) == cudaSuccess ? 1 : 0;
-      });
-      ldlt_inv_tile_kernel<128><<<1, TileChol<128>::NTHR, TileChol<128>::SMEM, s>>>(G, r, Ginv, gsplit, status);
-      break;
-    }
-    default: {
-      static std::atomic<int> attr[kMaxDevices];
-      per_device(attr, [] {
-        return cudaFuncSetAttribute(ldlt_inv_tile_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)TileChol<256>::SMEM) == cudaSuccess ? 1 : 0;
-      });
-      ldlt_inv_tile_kernel<256><<<1, TileChol<256>::NTHR, TileChol<256>::SMEM, s>>>(G, r, Ginv, nullptr, status);
-    }
+    case 16: return NMD_GI(16);
+    case 32: return NMD_GI(32);
+    case 64: return NMD_GI(64);
+  }
+#undef NMD_GI
+  return false;
+}
+
+void launch_chol_inv(const float* G, int r, int rp, float* Ginv, bf16* gsplit, int* status, cudaStream_t s) {
+  // (r_pad <= 64: launch_gram_inv)
+  static std::atomic<int> a128[kMaxDevices], a256[kMaxDevices];
+  if (rp == 128) {
+    per_device(a128, [] {
+      return cudaFuncSetAttribute(ldlt_inv_tile_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)TileChol<128>::SMEM) == cudaSuccess ? 1 : 0;
+    });
+    ldlt_inv_tile_kernel<128><<<1, TileChol<128>::NTHR, TileChol<128>::SMEM, s>>>(G, r, Ginv, gsplit, status);
+  } else {
+    per_device(a256, [] {
+      return cudaFuncSetAttribute(ldlt_inv_tile_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)TileChol<256>::SMEM) == cudaSuccess ? 1 : 0;
+    });
+    ldlt_inv_tile_kernel<256><<<1, TileChol<256>::NTHR, TileChol<256>::SMEM, s>>>(G, r, Ginv, nullptr, status);
   }
 }
 

@@ -128,7 +128,7 @@ struct Workspace {
   // added to R by the update; two copies like R
   float* Rs = nullptr;
   float* Rs2 = nullptr;
-  float* gram_part = nullptr;  // kGramParts x rp x rp
+  float* gram_part = nullptr;  // (kGramParts + 8) x rp x rp: the partials and the sums of their classes
   float* G = nullptr;          // rp x rp (Gram, for verification)
   float* Ginv = nullptr;       // rp x rp
   float* G2 = nullptr;
@@ -140,7 +140,8 @@ struct Workspace {
   double* loss_part = nullptr; // kLossParts x 8
   double* loss_out = nullptr;  // 8
   int* status = nullptr;       // kStatusWords
-  int* counters = nullptr;     // 64 ints; 0-1: skipped Delta-form chunks (u64), 2: deferred update's tiles
+  // 64 ints; 0-1: skipped Delta-form chunks (u64), 2: deferred update's tiles, 8-16: Gram chain
+  int* counters = nullptr;
   float* seg_partials = nullptr;  // max segments x rp (sparse correction of long rows)
   uint8_t* flags = nullptr;       // the panels' support-row flags, concatenated
   float* rpart = nullptr;         // kRpartRows x rp: partial R's of split-K steps
@@ -246,8 +247,14 @@ void launch_gram_reduce(const float* parts, int nparts, int r, int rp, float rid
 // both
 void launch_gram(const Factor* fq, bool rounded, int64_t q0, int64_t K, int r, int rp, float* parts, int nparts,
                  int64_t chunk, float ridge, float* G, cudaStream_t s);
-// Ginv = G^{-1} through the Cholesky (L D L^T) factorisation; NMD_ERR_NOT_SPD
-// in the status words on failure
+// r_pad <= 64: partials, G and G^{-1} in one launch (sums: 8 rp x rp floats of
+// scratch; ctr: 9 ints, zero between launches, one launch at a time).  False
+// for a larger rank.
+bool launch_gram_inv(const Factor* fq, bool rounded, int64_t q0, int64_t K, int r, int rp, float* parts, float* sums,
+                     int nparts, int64_t chunk, float ridge, float* G, float* Ginv, bf16* gsplit, int* ctr,
+                     int* status, cudaStream_t s);
+// r_pad >= 128: Ginv = G^{-1} through the Cholesky (L D L^T) factorisation;
+// NMD_ERR_NOT_SPD in the status words on failure
 // G^{-1} (rp x rp, row-major); with gsplit also its hi and lo bf16 pieces,
 // transposed (gsplit[n * split_stride(rp) + k] = hi(G^{-1}[k][n]), lo at
 // gsplit + rp * split_stride(rp)), pad entries zero
