@@ -9,6 +9,7 @@
 #include <atomic>
 
 #include "nmd_internal.cuh"
+#include "tc_ptx.cuh"
 
 namespace nmd {
 
@@ -1239,9 +1240,15 @@ __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& hi, uin
 // to the lanes of their slot by shuffles; an item's indices, values and m_i
 // are loaded while the previous item is computed, its descriptor two items
 // ahead.  In shared memory, 16-byte chunk j of row k sits at chunk j ^ ((k >>
-// 1) & (NCH - 1)).  Every index lies in [q0, q0 + K): the panel lists are
-// built at create from the CSR cut to the block's columns (rows, for row
-// steps), as for the kernels above.
+// 1) & (NCH - 1)); the lane that fetches an entry keeps its row's address with
+// that pattern, so that the address of a lane's chunk is one exclusive or away,
+// and entry slots past the item's end read a row of zeros behind the block (dot
+// product and coefficient 0) instead of being predicated.  What bounds it is
+// instruction issue (68% of the active cycles, shared memory and L2 well
+// below), so the address arithmetic counts: planted, r = 32, 2 M entries a
+// step, 38.8 us with indices, 35.8 us with addresses.  Every index lies in
+// [q0, q0 + K): the panel lists are built at create from the CSR cut to the
+// block's columns (rows, for row steps), as for the kernels above.
 // ---------------------------------------------------------------------------
 constexpr size_t kSparseQBytes = 200 * 1024;
 
@@ -1257,16 +1264,6 @@ __device__ __forceinline__ void unpack8(const uint4& u, float2* f) {
   const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
   for (int q = 0; q < 4; ++q) f[q] = make_float2(__uint_as_float(w[q] << 16), __uint_as_float(w[q] & 0xffff0000u));
-}
-
-// d = a b + c on a pair of floats (one packed fp32 FMA, each half rounded as fmaf)
-__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
-  float2 d;
-  asm("{.reg .b64 ra, rb, rc, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
-      "fma.rn.f32x2 rd, ra, rb, rc;\n\tmov.b64 {%0, %1}, rd;}"
-      : "=f"(d.x), "=f"(d.y)
-      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-  return d;
 }
 
 template <int RP>
@@ -1288,34 +1285,39 @@ __global__ void __launch_bounds__(32 * SpSmem<RP>::WARPS, 1) sparse_smem_kernel(
   cp_async_commit();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int ch = lane % NCH, slot = lane / NCH;
+  const uint32_t chx = (uint32_t)ch << 4;
   const int64_t nlong = nrows + nwhole, nitems = nlong + nseg;
   const int64_t stride = (int64_t)gridDim.x * C::WARPS;
   auto desc = [&](int64_t x) -> PanelRow {
     if (x >= nitems) return PanelRow{0, 0, 0};
     return x < nrows ? rows[x] : x < nlong ? whole[x - nrows] : seg[x - nlong];
   };
-  // an item's indices (relative to the block), values and this lane's chunk of m_i
-  auto fetch = [&](const PanelRow& pr, int* k4, float* s4, uint4& mc) {
+  // an item's row addresses in shared memory (see above), values and this
+  // lane's chunk of m_i
+  const uint32_t zrow = (uint32_t)K * (NCH * 16), qbase = (uint32_t)__cvta_generic_to_shared(qs);
+  auto fetch = [&](const PanelRow& pr, uint32_t* k4, float* s4, uint4& mc) {
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       const int e = lane + 32 * t;
       const bool live = e < pr.len;
-      k4[t] = live ? (int)(__ldg(qidx + pr.beg + e) - q0) : 0;
+      const uint32_t k = live ? (uint32_t)(__ldg(qidx + pr.beg + e) - (int32_t)q0) : 0u;
+      k4[t] = qbase + (live ? k * (NCH * 16) + (((k >> 1) & (NCH - 1)) << 4) : zrow);
       s4[t] = live ? __ldg(vals + pr.beg + e) : 0.f;
     }
     mc = pr.len > 0 ? __ldg(reinterpret_cast<const uint4*>(Mop + (int64_t)pr.row * RP) + ch) : make_uint4(0, 0, 0, 0);
   };
   int64_t w = (int64_t)blockIdx.x * C::WARPS + warp;
   PanelRow cur = desc(w), nxt = desc(w + stride);
-  int kk[4];
+  uint32_t kk[4];
   float ss[4];
   uint4 mc;
   fetch(cur, kk, ss, mc);
+  if (threadIdx.x < NCH) qs[K * NCH + threadIdx.x] = make_uint4(0, 0, 0, 0);
   cp_async_wait_0();
   __syncthreads();
   for (; w < nitems; w += stride) {
     const PanelRow after = desc(w + 2 * stride);
-    int kn[4];
+    uint32_t kn[4];
     float sn[4];
     uint4 mn;
     fetch(nxt, kn, sn, mn);
@@ -1328,11 +1330,12 @@ __global__ void __launch_bounds__(32 * SpSmem<RP>::WARPS, 1) sparse_smem_kernel(
       if (it * EPW >= cur.len) break;   // warp-uniform
       const int e = it * EPW + slot;
       constexpr int PER = 32 / EPW;       // iterations per batch of 32 entries
-      const int k = __shfl_sync(0xffffffffu, kk[it / PER], e & 31);
+      const uint32_t ka = __shfl_sync(0xffffffffu, kk[it / PER], e & 31);
       const float sv = __shfl_sync(0xffffffffu, ss[it / PER], e & 31);
-      const bool live = e < cur.len;
-      uint4 qc = make_uint4(0, 0, 0, 0);
-      if (live) qc = qs[k * NCH + (ch ^ ((k >> 1) & (NCH - 1)))];
+      uint4 qc;
+      asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                   : "=r"(qc.x), "=r"(qc.y), "=r"(qc.z), "=r"(qc.w)
+                   : "r"(ka ^ chx));
       float2 f[4];
       unpack8(qc, f);
       // the even and the odd columns' products summed separately, then added
@@ -1342,12 +1345,10 @@ __global__ void __launch_bounds__(32 * SpSmem<RP>::WARPS, 1) sparse_smem_kernel(
       float dot = d2.x + d2.y;
 #pragma unroll
       for (int o = 1; o < NCH; o <<= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-      if (live) {
-        const float cv = sv - fminf(0.f, dot);
-        const float2 c2 = make_float2(cv, cv);
+      const float cv = sv - fminf(0.f, dot);
+      const float2 c2 = make_float2(cv, cv);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q] = ffma2(c2, f[q], acc[q]);
-      }
+      for (int q = 0; q < 4; ++q) acc[q] = ffma2(c2, f[q], acc[q]);
     }
 #pragma unroll
     for (int o = NCH; o < 32; o <<= 1)
@@ -2291,12 +2292,12 @@ static bool launch_sparse_smem(const StepArgs& a, const PanelRow* rows, int64_t 
   static std::atomic<int> attr[kMaxDevices];
   if (!per_device(attr, [] {
         return cudaFuncSetAttribute(sparse_smem_kernel<RP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)kSparseQBytes) == cudaSuccess ? 1 : 0;
+                                    (int)kSparseQBytes + RP * (int)sizeof(bf16)) == cudaSuccess ? 1 : 0;
       }))
     return false;
   const int64_t nitems = nrows + nwhole + nseg;
   const int64_t grid = std::min<int64_t>(a.num_sms, (nitems + C::WARPS - 1) / C::WARPS);
-  const size_t smem = (size_t)a.K * RP * sizeof(bf16);
+  const size_t smem = (size_t)(a.K + 1) * RP * sizeof(bf16);   // the block and a row of zeros
   sparse_smem_kernel<RP><<<(unsigned)grid, 32 * C::WARPS, smem, s>>>(rows, nrows, whole, nwhole, seg, nseg, a.fm->hi,
                                                                     a.m0, a.fq->hi, a.q0, a.K, qidx, vals, R,
                                                                     partials);
