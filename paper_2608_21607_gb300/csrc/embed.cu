@@ -38,6 +38,11 @@ constexpr int kEmbedMaxRank = 128;   // xi has 2r <= 256 coordinates (the kernel
 // ordering gives n2 / 2 disjoint pairs, one warp per pair; a rotation with
 // t = tan(theta) = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)),
 // zeta = (|x_q|^2 - |x_p|^2) / (2 x_p . x_q), makes the pair orthogonal.
+// A step is a chain of latencies (two columns read, three sums, the rotation,
+// the columns written, a barrier), about 1,500 steps in all for r = 64: X and V
+// live in shared memory (128 KB at r = 128), and the eigendecompositions of G_A
+// and G_B run in two blocks at once.  (In global memory and one after the
+// other the core took most of the embedding's 3.75 ms at r = 64.)
 __device__ void jacobi(float* X, float* V, int n, volatile int* changed) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int n2 = n + (n & 1);
@@ -105,31 +110,41 @@ __device__ void column_norms(const float* X, int n, float* out) {
   }
 }
 
+// Block 0: X_A = G_A V_A with orthogonal columns, block 1: the same for G_B
+// (rp-strided rows; only the r x r part is read).  scr holds six r x r
+// matrices: X_A, V_A, X_B, V_B, C, V_C.
+__global__ void __launch_bounds__(1024) embed_eig_kernel(const float* __restrict__ GA, const float* __restrict__ GB,
+                                                         int r, int rp, float* __restrict__ scr) {
+  extern __shared__ __align__(16) float sme[];
+  __shared__ int changed;
+  const size_t rr = (size_t)r * r;
+  const float* G = blockIdx.x == 0 ? GA : GB;
+  float* X = sme;
+  float* V = sme + rr;
+  float* out = scr + (blockIdx.x == 0 ? 0 : 2 * rr);
+  for (int e = threadIdx.x; e < r * r; e += blockDim.x)   // symmetric: column-major = row-major
+    X[e] = G[(size_t)(e / r) * rp + e % r];
+  __syncthreads();
+  // G = P Lambda P^T: for a positive semi-definite G, G V has columns lambda_k p_k with V = P
+  jacobi(X, V, r, &changed);
+  for (int e = threadIdx.x; e < 2 * r * r; e += blockDim.x) out[e] = sme[e];
+}
+
 // T_A, T_B (r x r, row-major, columns in descending order of sigma) and sigma
-// from G_A, G_B (rp-strided rows; only the r x r part is read).  scr holds
-// six r x r matrices.
-__global__ void __launch_bounds__(1024) embed_core_kernel(const float* __restrict__ GA,
-                                                          const float* __restrict__ GB, int r, int rp,
-                                                          float* __restrict__ scr, float* __restrict__ TA,
+// from the eigendecompositions of embed_eig_kernel
+__global__ void __launch_bounds__(1024) embed_core_kernel(int r, float* __restrict__ scr, float* __restrict__ TA,
                                                           float* __restrict__ TB, float* __restrict__ sigma) {
+  extern __shared__ __align__(16) float sme[];
   __shared__ int changed;
   __shared__ float la[kEmbedMaxRank], lb[kEmbedMaxRank], sg[kEmbedMaxRank];
   __shared__ int rank[kEmbedMaxRank];
   const size_t rr = (size_t)r * r;
-  float* XA = scr;
-  float* VA = XA + rr;
-  float* XB = VA + rr;
-  float* VB = XB + rr;
-  float* C = VB + rr;
-  float* VC = C + rr;
-  for (int e = threadIdx.x; e < r * r; e += blockDim.x) {   // symmetric: column-major = row-major
-    XA[e] = GA[(size_t)(e / r) * rp + e % r];
-    XB[e] = GB[(size_t)(e / r) * rp + e % r];
-  }
-  __syncthreads();
-  // G = P Lambda P^T: for a positive semi-definite G, G V has columns lambda_k p_k with V = P
-  jacobi(XA, VA, r, &changed);
-  jacobi(XB, VB, r, &changed);
+  const float* XA = scr;
+  const float* VA = XA + rr;
+  const float* XB = VA + rr;
+  const float* VB = XB + rr;
+  float* C = sme;
+  float* VC = sme + rr;
   column_norms(XA, r, la);
   column_norms(XB, r, lb);
   __syncthreads();
@@ -291,17 +306,23 @@ nmd_status launch_embed(const Factor& W, const Factor& B, int64_t n, int r, int 
   const int64_t chunk = ((n + kGramParts - 1) / kGramParts + 31) / 32 * 32;
   launch_gram(&W, false, 0, n, r, rp, gram_part, kGramParts, chunk, 0.f, GA, s);
   launch_gram(&B, false, 0, n, r, rp, gram_part, kGramParts, chunk, 0.f, GB, s);
-  embed_core_kernel<<<1, 1024, 0, s>>>(GA, GB, r, rp, scratch, TA, TB, sigma);
   static std::atomic<int> attr[kMaxDevices];
   if (!per_device(attr, [] {
-        return cudaFuncSetAttribute(embed_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)(2 * kEmbedMaxRank * kEmbedMaxRank * sizeof(float))) == cudaSuccess ? 1 : 0;
+        constexpr int most = (int)(2 * kEmbedMaxRank * kEmbedMaxRank * sizeof(float));
+        return cudaFuncSetAttribute(embed_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most) ==
+                           cudaSuccess &&
+                       cudaFuncSetAttribute(embed_eig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most) ==
+                           cudaSuccess &&
+                       cudaFuncSetAttribute(embed_core_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most) ==
+                           cudaSuccess ? 1 : 0;
       }))
     return NMD_ERR_CUDA;
   const size_t smem = (size_t)2 * r * r * sizeof(float);
+  embed_eig_kernel<<<2, 1024, smem, s>>>(GA, GB, r, rp, scratch);
+  embed_core_kernel<<<1, 1024, smem, s>>>(r, scratch, TA, TB, sigma);
   const unsigned grid = (unsigned)std::min<int64_t>((n + 7) / 8, (int64_t)num_sms * 4);
   embed_rows_kernel<<<grid, 256, smem, s>>>(W.master, B.master, n, r, rp, TA, TB, xi);
-  *launches += 6;
+  *launches += 7;
   return NMD_OK;
 }
 
