@@ -123,9 +123,9 @@ struct Cfg {
   static constexpr size_t OFF_W = (size_t)NSTAGE * STAGE_BYTES;
   static constexpr int W_PANEL_BYTES = BM * ROWB;     // one swizzle panel of a W tile
   static constexpr size_t OFF_STG = OFF_W + (size_t)NWB * W_BYTES;
-  // loss pass: each epilogue thread's window of column indices (16, at a stride of 17)
+  // loss pass: each epilogue thread's window of column indices (32, at a stride of 33)
   static constexpr size_t OFF_WIN = OFF_STG;
-  static constexpr int WIN_BYTES = LOSS ? kEpiThreads * 17 * 4 : 0;
+  static constexpr int WIN_BYTES = LOSS ? kEpiThreads * 33 * 4 : 0;
   static constexpr size_t OFF_BARS = OFF_STG + STG_BYTES + WIN_BYTES;
   static constexpr int COL_L = 0;                     // NB x BN columns
   static constexpr int COL_R = NB * BN;               // NRB x RCOLS columns
@@ -661,11 +661,11 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
         pready = __all_sync(0xffffffffu, pr);
       }
     } else {
+      // (a chunk's barriers are tested while the chunk before is issued)
+      bool ready = false;
       while (k1.valid()) {
-        const bool ready = mbar_test_wait(b_full + 8 * s1, ph_full) & mbar_test_wait(b_lfree + 8 * l1, ph_lfree);
-        if (!__all_sync(0xffffffffu, ready) &&
-            (!conv_wait(b_full + 8 * s1, ph_full, abort_flag, p.status, 3) ||
-             !conv_wait(b_lfree + 8 * l1, ph_lfree, abort_flag, p.status, 4)))
+        if (!ready && (!conv_wait(b_full + 8 * s1, ph_full, abort_flag, p.status, 3) ||
+                       !conv_wait(b_lfree + 8 * l1, ph_lfree, abort_flag, p.status, 4)))
           break;
         if (k1.first) {
           if (!conv_wait(b_wfull + 8 * wb1, ph_wfull, abort_flag, p.status, 2)) break;
@@ -674,11 +674,14 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
         }
         fence_after();
         const bool last = k1.last();
-        mma1(s1, l1, wb1);
-        commit_elect(b_lfull + 8 * l1);
-        if (LOSS) commit_elect(b_empty + 8 * s1);
-        if (last) commit_elect(b_wempty + 8 * wb1);
+        const int s = s1, l = l1, wb = wb1;
         advance1(last);
+        const bool next = mbar_test_wait(b_full + 8 * s1, ph_full) & mbar_test_wait(b_lfree + 8 * l1, ph_lfree);
+        mma1(s, l, wb);
+        commit_elect(b_lfull + 8 * l);
+        if (LOSS) commit_elect(b_empty + 8 * s);
+        if (last) commit_elect(b_wempty + 8 * wb);
+        ready = __all_sync(0xffffffffu, next);
       }
     }
     // wait until every MMA issued by this warp has completed
@@ -738,9 +741,10 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
     bool ok = true;
     // loss pass: this thread's row of S, walked alongside the column chunks so
     // that support entries are left to the support pass (no cancellation)
-    constexpr int kWin = 16;
+    constexpr int kWin = 32;
     int64_t se = 0, send = 0;              // the row's entries from the window's first to its last
     int wpos = 0, wcnt = 0;                // position in the window, entries in it
+    int64_t snext = INT_MAX;               // the next entry's column (see support_mask)
     int* win = (int*)(smem + C::OFF_WIN) + et * (kWin + 1);
 
     // load the W tile `tile` into W buffer wb: warpgroup g takes 8-word groups g, g+2, ...
@@ -804,53 +808,59 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
       if (lane == 0) mbar_arrive(b_wfull + 8 * wb);
     };
 
-    // Loss pass: this row's entries in columns [c0, c0 + BN) as bits, c0
-    // ascending within a tile.  The row's next entries sit in a window of
-    // kWin column indices in shared memory (a dependent global load per entry
-    // held the epilogue up for most of the pass: 8.1 ms at 139,255 nodes and 2.8M
-    // entries), refilled by the row's own thread, its loads in flight
-    // together.  A row that needs more than one refill within a chunk (a hub
-    // of the graph has an entry in every column) is read on by the whole
-    // warp, 256 entries at a time.  Called by converged warps.
+    // Loss pass: this row's entries in columns [c0, c0 + BN) as bits (bit b of
+    // m0: column c0 + b, of m1: c0 + 64 + b), c0 ascending within a tile.  The
+    // row's next entries sit in a window of kWin column indices in shared memory
+    // (a dependent global load per entry held the epilogue up for most of the
+    // pass), refilled by the row's own thread, its loads in flight together; the
+    // next column is kept in a register, so that a warp without an entry in the
+    // chunk passes on after one vote.  Where few rows need more entries than
+    // their windows hold, the whole warp reads on in each, 256 entries at a time;
+    // a row with many entries per chunk (a hub of the graph has one in every
+    // column) is left without a window and read that way in every chunk.
+    // Called by converged warps.
     auto refill = [&](int64_t from) {   // this thread's window: entries [from, from + kWin) of its row
       se = from;
       wpos = 0;
       wcnt = (int)(send - from < kWin ? send - from : kWin);
-      int col[kWin];
+      for (int h = 0; h < wcnt; h += 16) {
+        int col[16];
 #pragma unroll
-      for (int i = 0; i < kWin; ++i) col[i] = i < wcnt ? p.cidx[from + i] : 0;
+        for (int i = 0; i < 16; ++i) col[i] = h + i < wcnt ? p.cidx[from + h + i] : 0;
 #pragma unroll
-      for (int i = 0; i < kWin; ++i) win[i] = col[i];
+        for (int i = 0; i < 16; ++i) win[h + i] = col[i];
+      }
+      snext = wcnt > 0 ? win[0] : INT_MAX;
     };
-    auto support_mask = [&](int64_t c0, uint32_t(&msk)[BN / 32]) {
-      constexpr int W = BN / 32;
+    auto set_bit = [](uint64_t& m0, uint64_t& m1, int b) {
+      const uint64_t bit = 1ull << (b & 63);
+      m0 |= b < 64 ? bit : 0ull;
+      m1 |= b < 64 ? 0ull : bit;
+    };
+    auto support_mask = [&](int64_t c0, uint64_t& m0, uint64_t& m1) {
+      m0 = m1 = 0ull;
       const int64_t cend = c0 + BN;
-#pragma unroll
-      for (int w = 0; w < W; ++w) msk[w] = 0u;
-      for (int pass = 0;; ++pass) {
-        for (; wpos < wcnt; ++wpos) {
-          const int64_t col = win[wpos];
-          if (col >= cend) break;
-          const int b = (int)(col - c0);
-#pragma unroll
-          for (int w = 0; w < W; ++w)
-            if (b >= 0 && w == (b >> 5)) msk[w] |= 1u << (b & 31);
+      // snext: the next column; INT_MIN: more entries, not in the window; INT_MAX: none
+      while (__any_sync(0xffffffffu, snext < cend)) {
+        while (snext < cend && snext != INT_MIN) {
+          const int b = (int)(snext - c0);
+          if (b >= 0) set_bit(m0, m1, b);
+          ++wpos;
+          snext = wpos < wcnt ? win[wpos] : se + wcnt < send ? INT_MIN : INT_MAX;
         }
-        const bool out = wpos == wcnt && se + wcnt < send;   // the window is used up, the row is not
-        uint32_t more = __ballot_sync(0xffffffffu, out);
-        if (more == 0u) break;
-        if (pass == 0 || __popc(more) > 4) {
-          if (out) refill(se + wcnt);
+        __syncwarp();
+        uint32_t more = __ballot_sync(0xffffffffu, snext == INT_MIN);
+        if (__popc(more) > 4) {
+          if (snext == INT_MIN) refill(se + wcnt);
+          __syncwarp();
           continue;
         }
         while (more) {
           const int src = __ffs(more) - 1;
           more &= more - 1;
           int64_t q = __shfl_sync(0xffffffffu, se + wcnt, src);
-          const int64_t e = __shfl_sync(0xffffffffu, send, src);
-          uint32_t m[W];
-#pragma unroll
-          for (int w = 0; w < W; ++w) m[w] = 0u;
+          const int64_t e = __shfl_sync(0xffffffffu, send, src), q0 = q;
+          uint64_t a0 = 0ull, a1 = 0ull;
           int n;
           do {
             int col[8];
@@ -859,24 +869,34 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
             n = 0;
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
-              const bool in = col[k] < cend && col[k] != INT_MAX;
-              n += __popc(__ballot_sync(0xffffffffu, in));
-              const int64_t b = (int64_t)col[k] - c0;
-              if (__any_sync(0xffffffffu, in && b >= 0))
-#pragma unroll
-                for (int w = 0; w < W; ++w)
-                  m[w] |= __reduce_or_sync(0xffffffffu, in && b >= 0 && (int)(b >> 5) == w ? 1u << ((int)b & 31) : 0u);
+              const bool in = col[k] < cend;   // (columns lie below INT_MAX)
+              n += __popc(__ballot_sync(0xffffffffu, in && col[k] != INT_MAX));
+              if (in && col[k] != INT_MAX && col[k] >= c0) set_bit(a0, a1, (int)(col[k] - c0));
             }
             q += n;
           } while (n == 256);
-          if (lane == src) {
 #pragma unroll
-            for (int w = 0; w < W; ++w) msk[w] |= m[w];
-            refill(q);
+          for (int w = 0; w < 2; ++w) {
+            const uint64_t a = w ? a1 : a0;
+            const uint64_t all = ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(a >> 32)) << 32) |
+                                 __reduce_or_sync(0xffffffffu, (uint32_t)a);
+            if (lane == src) {
+              if (w) m1 |= all;
+              else m0 |= all;
+            }
+          }
+          if (lane == src) {
+            if (q - q0 >= 16 && q < e) {   // no window: the warp reads on in the next chunk
+              se = q;
+              wpos = wcnt = 0;
+              snext = INT_MIN;
+            } else {
+              refill(q);
+            }
           }
           __syncwarp();
         }
-        break;   // those rows' windows now start past the chunk, or their rows end
+        break;   // those rows go on past the chunk, or end
       }
     };
 
@@ -917,9 +937,9 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
         odd = !odd;
         if (!C::HALF && odd != (wg != 0)) continue;
         // the support columns of this chunk, one bit each, found while the
-        // chunk's product is under way: bit i of msk[g] = column 32 g + i
-        uint32_t msk[BN / 32];
-        if (SUMS) support_mask(c * BN, msk);
+        // chunk's product is under way
+        uint64_t m0 = 0ull, m1 = 0ull;
+        if (SUMS) support_mask(c * BN, m0, m1);
         if (!(ok = conv_wait(b_lfull + 8 * lb, lpar, abort_flag, p.status, 7))) break;
         fence_after();
         const int kv = (int)(kK - c * BN < BN ? kK - c * BN : BN);   // valid columns in this chunk
@@ -962,7 +982,7 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
         // the first-product passes: one group of 32 columns, columns past the
         // Q side masked
         auto group = [&](uint32_t(&v)[32], int g) {
-          if (kv < BN) {
+          if (!NEAREST && kv < BN) {
 #pragma unroll
             for (int i = 0; i < 32; ++i)
               if (g * 32 + i >= kv) v[i] = 0u;
@@ -999,31 +1019,47 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
               for (int k = 0; k < 4; ++k) hrow[k] = make_uint4(hw[4 * k], hw[4 * k + 1], hw[4 * k + 2], hw[4 * k + 3]);
               if (!finite) record(p.status, NMD_ERR_DIVERGED, (int)(p.upd_row0 + li));
             }
-          } else if (NEAREST) {   // columns past the set or the row itself do not count
+          } else if (NEAREST) {
+            // columns past the set or the row itself do not count; the group's
+            // largest value first, its (first) place only where it beats the
+            // row's best so far
             const int64_t cb = c * BN + g * 32, self = (int64_t)t * BM + row;
+            if (kv < BN || (self >= cb && self < cb + 32)) {
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              const float x = __uint_as_float(v[i]);
-              if (g * 32 + i < kv && cb + i != self && x > nbest) {
-                nbest = x;
-                nidx = cb + i;
+              for (int i = 0; i < 32; ++i)
+                if (g * 32 + i >= kv || cb + i == self) v[i] = 0xff800000u;   // -inf
+            }
+            float gm = __uint_as_float(v[0]);
+#pragma unroll
+            for (int i = 1; i < 32; ++i) gm = fmaxf(gm, __uint_as_float(v[i]));
+            if (gm > nbest) {
+              bool found = false;
+#pragma unroll
+              for (int i = 0; i < 32; ++i) {
+                if (!found && __uint_as_float(v[i]) == gm) {
+                  found = true;
+                  nbest = __uint_as_float(v[i]);
+                  nidx = cb + i;
+                }
               }
             }
           } else if (SUMS) {
-            uint32_t mg = 0u;
-#pragma unroll
-            for (int w = 0; w < BN / 32; ++w) mg = w == g ? msk[w] : mg;
-            if (mg != 0u) {   // support columns in this group: zero them
+            const uint32_t mg = (uint32_t)((g < 2 ? m0 : m1) >> (32 * (g & 1)));
+            if (__any_sync(0xffffffffu, mg != 0u)) {   // support columns in this group: zero them
 #pragma unroll
               for (int i = 0; i < 32; ++i)
                 if ((mg >> i) & 1u) v[i] = 0u;
             }
+            // on t = x + |x| = 2 max(0, x) (exact, and at the full rate of the
+            // fp32 adds, which a maximum is not): c2 and c1 are 4 and 2 times the
+            // chunk's sums, rounded alike
 #pragma unroll
             for (int i = 0; i < 32; i += 2) {
-              const float x0 = fmaxf(0.f, __uint_as_float(v[i])), x1 = fmaxf(0.f, __uint_as_float(v[i + 1]));
-              c2 = fmaf(x0, x0, c2);
-              c2 = fmaf(x1, x1, c2);
-              c1 += x0 + x1;
+              const float x0 = __uint_as_float(v[i]), x1 = __uint_as_float(v[i + 1]);
+              const float t0 = x0 + fabsf(x0), t1 = x1 + fabsf(x1);
+              c2 = fmaf(t0, t0, c2);
+              c2 = fmaf(t1, t1, c2);
+              c1 += t0 + t1;
             }
           }
         };
@@ -1064,21 +1100,23 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
             }
           }
         } else {
+          // groups of 32 columns, the next one's load in flight while one is taken
+          uint32_t va[32], vb[32];
+          tmem_ld32(lcol, va);
 #pragma unroll 1
-          for (int jj = 0; jj < BN / 64; ++jj) {   // two groups per pass, both loads in flight
-            uint32_t v0[32], v1[32];
-            tmem_ld32(lcol + jj * 64, v0);
-            tmem_ld32(lcol + jj * 64 + 32, v1);
-            tmem_wait_ld(v0);
-            tmem_wait_ld(v1);
-            group(v0, 2 * jj);
-            group(v1, 2 * jj + 1);
+          for (int q = 0; q < BN / 32; q += 2) {
+            tmem_wait_ld(va);
+            tmem_ld32(lcol + q * 32 + 32, vb);
+            group(va, q);
+            tmem_wait_ld(vb);
+            if (q + 2 < BN / 32) tmem_ld32(lcol + q * 32 + 64, va);
+            group(vb, q + 1);
           }
         }
         if (LOSS) {
           if (SUMS) {
-            s2 += (double)c2;
-            s1 += (double)c1;
+            s2 += (double)(0.25f * c2);
+            s1 += (double)(0.5f * c1);
           }
           fence_before();
           __syncwarp();
