@@ -735,7 +735,16 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
     const int row = (warp & 3) * 32 + lane;
     const int et = threadIdx.x;                          // 0 .. 255
     const uint32_t lane_base = ((uint32_t)((warp & 3) * 32)) << 16;
+    // (loss) the chunks' sums of a row, as an fp32 sum and its rounding errors
+    // (exact but for the errors' own sum, 2^-48); fp64 adds, two a chunk and
+    // thread, cost more than the pass's tensor work.  Per tile into fp64.
     double s2 = 0.0, s1 = 0.0;
+    float h2 = 0.f, l2 = 0.f, h1 = 0.f, l1 = 0.f;
+    auto two_sum = [](float& h, float& l, float x) {
+      const float t = h + x, z = t - h;
+      l += (h - (t - z)) + (x - z);
+      h = t;
+    };
     float nbest = -INFINITY;   // nearest-neighbour pass: this thread's best L of its row so far
     int64_t nidx = -1;
     bool ok = true;
@@ -944,7 +953,7 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
         fence_after();
         const int kv = (int)(kK - c * BN < BN ? kK - c * BN : BN);   // valid columns in this chunk
         const uint32_t lcol = tmem + lane_base + C::COL_L + lb * BN;
-        float c2 = 0.f, c1 = 0.f;
+        float2 c2a = make_float2(0.f, 0.f), c2b = c2a, c1 = c2a;   // (loss) sums of relu(x)^2 and of relu(x)
         uint32_t nzacc = 0u;   // Delta form: OR of this thread's P words
         // MODE 0: P of one group of 32 columns of L (TMEM columns [32 g, 32 g + 32)
         // of the buffer): bf16, 16 TMEM columns at 16 g (HALF: within the
@@ -1050,16 +1059,15 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
               for (int i = 0; i < 32; ++i)
                 if ((mg >> i) & 1u) v[i] = 0u;
             }
-            // on t = x + |x| = 2 max(0, x) (exact, and at the full rate of the
-            // fp32 adds, which a maximum is not): c2 and c1 are 4 and 2 times the
-            // chunk's sums, rounded alike
+            // pairs of columns in packed FMAs, in two chains: one fp32 chain of
+            // 128 dependent FMAs a chunk set the pace of this loop
 #pragma unroll
-            for (int i = 0; i < 32; i += 2) {
-              const float x0 = __uint_as_float(v[i]), x1 = __uint_as_float(v[i + 1]);
-              const float t0 = x0 + fabsf(x0), t1 = x1 + fabsf(x1);
-              c2 = fmaf(t0, t0, c2);
-              c2 = fmaf(t1, t1, c2);
-              c1 += t0 + t1;
+            for (int i = 0; i < 32; i += 4) {
+              const float2 ta = make_float2(fmaxf(0.f, __uint_as_float(v[i])), fmaxf(0.f, __uint_as_float(v[i + 1])));
+              const float2 tb = make_float2(fmaxf(0.f, __uint_as_float(v[i + 2])), fmaxf(0.f, __uint_as_float(v[i + 3])));
+              c2a = ffma2(ta, ta, c2a);
+              c2b = ffma2(tb, tb, c2b);
+              c1 = fadd2(c1, fadd2(ta, tb));
             }
           }
         };
@@ -1115,8 +1123,8 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
         }
         if (LOSS) {
           if (SUMS) {
-            s2 += (double)(0.25f * c2);
-            s1 += (double)(0.5f * c1);
+            two_sum(h2, l2, (c2a.x + c2b.x) + (c2a.y + c2b.y));
+            two_sum(h1, l1, c1.x + c1.y);
           }
           fence_before();
           __syncwarp();
@@ -1138,6 +1146,11 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
         }
       }
       if (!ok) break;
+      if (SUMS) {
+        s2 += (double)h2 + (double)l2;
+        s1 += (double)h1 + (double)l1;
+        h2 = l2 = h1 = l1 = 0.f;
+      }
       if (NEAREST) {   // this warpgroup's best of the row; the two are merged by atomicMax
         const int64_t li = (int64_t)t * BM + row;
         if (li < p.M && nidx >= 0) {
