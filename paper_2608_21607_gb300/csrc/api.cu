@@ -320,7 +320,7 @@ void layout(Carver& c, int64_t m, int64_t n, int64_t nnz, int rp, int64_t npanel
   w->loss_part = c.take<double>((size_t)kLossParts * 8);
   w->loss_out = c.take<double>(8);
   w->status = c.take<int>(kStatusWords);
-  w->counters = c.take<int>(64);
+  w->counters = c.take<int>(kCounters);
   c.off = (c.off + 255) & ~size_t(255);
   w->bytes = c.off;
 }
@@ -545,7 +545,7 @@ Span panel_span(const Roles& ro) {
 
 nmd_status launch_span(nmd_handle* h, const StepArgs& a, const Roles& ro, const Span& sp, float* Rs, cudaStream_t s) {
   h->launches += launch_sparse(a, sp.rows, sp.nrows, sp.whole, sp.nwhole, sp.seg, sp.nseg, sp.multi, sp.nmulti,
-                               ro.qidx, ro.vals, Rs, h->ws.seg_partials, sp.seg_first, s);
+                               ro.qidx, ro.vals, Rs, h->ws.seg_partials, sp.seg_first, h->ws.counters + 64, s);
   return NMD_OK;
 }
 
@@ -1067,7 +1067,7 @@ nmd_status nmd_create(int64_t m, int64_t n, int32_t r, const int64_t* row_ptr,
   e = cudaMemsetAsync(h->ws.status, 0, kStatusWords * sizeof(int), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->ws.Rs, 0, std::max(m, n) * h->rp * sizeof(float), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->ws.Rs2, 0, std::max(m, n) * h->rp * sizeof(float), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->ws.counters, 0, 64 * sizeof(int), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->ws.counters, 0, kCounters * sizeof(int), s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return bail(NMD_ERR_CUDA, std::string("create: ") + cudaGetErrorString(e));
   // the host copies of the panel lists are kept for nmd_panel_traversal

@@ -1238,8 +1238,12 @@ __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& hi, uin
 // the slots and written once.  Each lane fetches one of every 32 entries'
 // index and value (at most 128 entries per item: four), and they are passed
 // to the lanes of their slot by shuffles; an item's indices, values and m_i
-// are loaded while the previous item is computed, its descriptor two items
-// ahead.  In shared memory, 16-byte chunk j of row k sits at chunk j ^ ((k >>
+// are loaded while the previous item is computed.  A warp's first two items go
+// round the blocks, the others are taken by count: a block that starts late,
+// behind a dense CTA with a second tile, takes fewer (planted, 157 tiles for
+// 152 SMs: 1,295 -> 1,142 us a sweep).  (kItemCounts counters kItemStride ints
+// apart, each over every kItemCounts-th item, as one for all costs 2 us; then
+// one of the blocks that are done, the last of which sets all to zero.)  In shared memory, 16-byte chunk j of row k sits at chunk j ^ ((k >>
 // 1) & (NCH - 1)); the lane that fetches an entry keeps its row's address with
 // that pattern, so that the address of a lane's chunk is one exclusive or away,
 // and entry slots past the item's end read a row of zeros behind the block (dot
@@ -1271,7 +1275,7 @@ __global__ void __launch_bounds__(32 * SpSmem<RP>::WARPS, 1) sparse_smem_kernel(
     const PanelRow* __restrict__ rows, int64_t nrows, const PanelRow* __restrict__ whole, int64_t nwhole,
     const PanelRow* __restrict__ seg, int64_t nseg, const bf16* __restrict__ Mop, int64_t m0,
     const bf16* __restrict__ Qop, int64_t q0, int64_t K, const int32_t* __restrict__ qidx,
-    const float* __restrict__ vals, float* __restrict__ R, float* __restrict__ partials) {
+    const float* __restrict__ vals, float* __restrict__ R, float* __restrict__ partials, int* __restrict__ ctr) {
   using C = SpSmem<RP>;
   constexpr int NCH = C::NCH, EPW = C::EPW;
   static_assert(RP == 16 || RP == 32, "r_pad 16 or 32");
@@ -1306,8 +1310,11 @@ __global__ void __launch_bounds__(32 * SpSmem<RP>::WARPS, 1) sparse_smem_kernel(
     }
     mc = pr.len > 0 ? __ldg(reinterpret_cast<const uint4*>(Mop + (int64_t)pr.row * RP) + ch) : make_uint4(0, 0, 0, 0);
   };
-  int64_t w = (int64_t)blockIdx.x * C::WARPS + warp;
-  PanelRow cur = desc(w), nxt = desc(w + stride);
+  int64_t w = (int64_t)warp * gridDim.x + blockIdx.x, wn = w + stride;
+  PanelRow cur = desc(w), nxt = desc(wn);
+  const int nc = min((int)gridDim.x, kItemCounts), cs = blockIdx.x % nc;
+  const bool count = nitems > 2 * stride;
+  int taken = 0;
   uint32_t kk[4];
   float ss[4];
   uint4 mc;
@@ -1315,8 +1322,8 @@ __global__ void __launch_bounds__(32 * SpSmem<RP>::WARPS, 1) sparse_smem_kernel(
   if (threadIdx.x < NCH) qs[K * NCH + threadIdx.x] = make_uint4(0, 0, 0, 0);
   cp_async_wait_0();
   __syncthreads();
-  for (; w < nitems; w += stride) {
-    const PanelRow after = desc(w + 2 * stride);
+  while (w < nitems) {
+    if (count && lane == 0) taken = atomicAdd(ctr + cs * kItemStride, 1);
     uint32_t kn[4];
     float sn[4];
     uint4 mn;
@@ -1350,18 +1357,28 @@ __global__ void __launch_bounds__(32 * SpSmem<RP>::WARPS, 1) sparse_smem_kernel(
 #pragma unroll
       for (int q = 0; q < 4; ++q) acc[q] = ffma2(c2, f[q], acc[q]);
     }
+    const int64_t wa = 2 * stride + cs + (int64_t)nc * __shfl_sync(0xffffffffu, taken, 0);
+    const PanelRow after = desc(wa);
+    // the slots' sums: each exchange halves the columns a lane still holds
+    float v[8] = {acc[0].x, acc[0].y, acc[1].x, acc[1].y, acc[2].x, acc[2].y, acc[3].x, acc[3].y};
+    int col = 8 * ch;
 #pragma unroll
-    for (int o = NCH; o < 32; o <<= 1)
+    for (int o = NCH, n = 4; o < 32; o <<= 1, n >>= 1) {
+      if (n == 0) {
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+      } else {
+        const bool up = (lane & o) != 0;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        acc[q].x += __shfl_xor_sync(0xffffffffu, acc[q].x, o);
-        acc[q].y += __shfl_xor_sync(0xffffffffu, acc[q].y, o);
+        for (int q = 0; q < n; ++q) {
+          const float send = up ? v[q] : v[n + q], keep = up ? v[n + q] : v[q];
+          v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+        col += up ? n : 0;
       }
-    if (slot == 0) {
-      float* out = (w < nlong ? R + ((int64_t)cur.row - m0) * RP : partials + (w - nlong) * RP) + 8 * ch;
-      *(float4*)out = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
-      *(float4*)(out + 4) = make_float4(acc[2].x, acc[2].y, acc[3].x, acc[3].y);
     }
+    if (lane < RP) (w < nlong ? R + ((int64_t)cur.row - m0) * RP : partials + (w - nlong) * RP)[col] = v[0];
+    w = wn;
+    wn = wa;
     cur = nxt;
     nxt = after;
     mc = mn;
@@ -1370,6 +1387,14 @@ __global__ void __launch_bounds__(32 * SpSmem<RP>::WARPS, 1) sparse_smem_kernel(
       kk[t] = kn[t];
       ss[t] = sn[t];
     }
+  }
+  // the last block leaves the counts at zero for the next launch
+  if (!count) return;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(ctr + kItemCounts * kItemStride, 1) == (int)gridDim.x - 1)
+      for (int c = 0; c <= kItemCounts; ++c) ctr[c * kItemStride] = 0;
   }
 }
 
@@ -2287,7 +2312,7 @@ static void launch_reduce(const PanelRow* multi, int64_t nmulti, const float* pa
 template <int RP>
 static bool launch_sparse_smem(const StepArgs& a, const PanelRow* rows, int64_t nrows, const PanelRow* whole,
                                int64_t nwhole, const PanelRow* seg, int64_t nseg, const int32_t* qidx,
-                               const float* vals, float* R, float* partials, cudaStream_t s) {
+                               const float* vals, float* R, float* partials, int* ctr, cudaStream_t s) {
   using C = SpSmem<RP>;
   static std::atomic<int> attr[kMaxDevices];
   if (!per_device(attr, [] {
@@ -2300,13 +2325,13 @@ static bool launch_sparse_smem(const StepArgs& a, const PanelRow* rows, int64_t 
   const size_t smem = (size_t)(a.K + 1) * RP * sizeof(bf16);   // the block and a row of zeros
   sparse_smem_kernel<RP><<<(unsigned)grid, 32 * C::WARPS, smem, s>>>(rows, nrows, whole, nwhole, seg, nseg, a.fm->hi,
                                                                     a.m0, a.fq->hi, a.q0, a.K, qidx, vals, R,
-                                                                    partials);
+                                                                    partials, ctr);
   return true;
 }
 
 int launch_sparse(const StepArgs& a, const PanelRow* rows, int64_t nrows, const PanelRow* whole, int64_t nwhole,
                   const PanelRow* seg, int64_t nseg, const PanelRow* multi, int64_t nmulti, const int32_t* qidx,
-                  const float* vals, float* R, float* partials, int64_t seg_first, cudaStream_t s) {
+                  const float* vals, float* R, float* partials, int64_t seg_first, int* ctr, cudaStream_t s) {
   // slice w of `seg` is slice seg_first + w of its block, whose partial slot
   // the reduction (multi[].beg, relative to the block) reads
   float* seg_partials = partials + seg_first * a.rp;
@@ -2314,9 +2339,9 @@ int launch_sparse(const StepArgs& a, const PanelRow* rows, int64_t nrows, const 
   if (a.precision == NMD_BF16 && (a.rp == 16 || a.rp == 32) && a.K * a.rp * 2 <= (int64_t)kSparseQBytes &&
       nrows + nwhole + nseg > 0) {
     const bool ok = a.rp == 16 ? launch_sparse_smem<16>(a, rows, nrows, whole, nwhole, seg, nseg, qidx, vals, R,
-                                                        seg_partials, s)
+                                                        seg_partials, ctr, s)
                                : launch_sparse_smem<32>(a, rows, nrows, whole, nwhole, seg, nseg, qidx, vals, R,
-                                                        seg_partials, s);
+                                                        seg_partials, ctr, s);
     if (ok) {
       if (nseg > 0) launch_reduce(multi, nmulti, partials, R, a.m0, a.rp, s);
       return 1 + (nseg > 0);

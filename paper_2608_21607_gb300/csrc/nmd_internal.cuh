@@ -140,7 +140,8 @@ struct Workspace {
   double* loss_part = nullptr; // kLossParts x 8
   double* loss_out = nullptr;  // 8
   int* status = nullptr;       // kStatusWords
-  // 64 ints; 0-1: skipped Delta-form chunks (u64), 2: deferred update's tiles, 8-16: Gram chain
+  // kCounters ints; 0-1: skipped Delta-form chunks (u64), 2: deferred update's tiles, 8-16: Gram chain,
+  // 64-: support term's items (kItemCounts + 1, kItemStride apart)
   int* counters = nullptr;
   float* seg_partials = nullptr;  // max segments x rp (sparse correction of long rows)
   uint8_t* flags = nullptr;       // the panels' support-row flags, concatenated
@@ -167,6 +168,8 @@ struct Workspace {
 constexpr int split_stride(int rp) { return rp + 8; }
 
 constexpr int kGramParts = 64;
+constexpr int kItemCounts = 8, kItemStride = 32;   // support term: counters of taken items, ints between them
+constexpr int kCounters = 64 + (kItemCounts + 1) * kItemStride;
 constexpr int64_t kRpartRows = 256 * 128;   // splits x tiles x 128 rows never exceed 256 SMs' worth
 constexpr int kLossParts = 2048;
 
@@ -265,10 +268,11 @@ void launch_small_gemm(const float* A, int64_t lda, const float* B, int64_t ldb,
 // rows: short rows; whole: the whole rows of the long-row kernel; seg: the
 // slices of the split rows, summed per row of `multi` into R
 // (bf16 mode: the factors' hi pieces, else the fp32 masters)
-// returns the number of kernels launched
+// returns the number of kernels launched; ctr: (kItemCounts + 1)
+// kItemStride ints, zero between launches, one launch at a time
 int launch_sparse(const StepArgs& a, const PanelRow* rows, int64_t nrows, const PanelRow* whole,
                    int64_t nwhole, const PanelRow* seg, int64_t nseg, const PanelRow* multi, int64_t nmulti,
-                   const int32_t* qidx, const float* vals, float* R, float* partials, int64_t seg_first,
+                   const int32_t* qidx, const float* vals, float* R, float* partials, int64_t seg_first, int* ctr,
                    cudaStream_t s);
 // flags: one byte per row of the step (Rs is read only where it is nonzero)
 // gsplit: G^{-1}'s pieces as written by launch_chol_inv (read by the bf16
