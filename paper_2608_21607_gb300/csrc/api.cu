@@ -1103,24 +1103,41 @@ nmd_status copy_split(nmd_handle* h, void* dst, const void* src, size_t bytes, c
   return NMD_OK;
 }
 
+// Whether kernels on the handle's device may access p: memory of that device
+// or managed memory; anything else is staged by copies.
+bool readable_here(const nmd_handle* h, const void* p) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return (at.type == cudaMemoryTypeDevice && at.device == h->device) || at.type == cudaMemoryTypeManaged;
+}
+
 nmd_status nmd_set_factors(nmd_handle* h, const float* W, const float* H, int on_device) {
   if (!h || !W || !H) return fail(h, NMD_ERR_INVALID, "NULL argument to nmd_set_factors");
   DeviceScope dg(h);
   h->fver[0]++;
   h->fver[1]++;
   cudaStream_t s = h->stream;
-  cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  // stage through R (max(m, n) x rp floats >= m x r and r x n)
-  nmd_status cs = copy_split(h, h->ws.R, W, (size_t)h->m * h->r * 4, kind, s);
-  if (cs != NMD_OK) return cs;
-  launch_pack(h->ws.R, false, h->m, h->r, h->rp, h->W, s);
-  h->launches++;
-  // H goes to the second copy of R, so that its copy overlaps W's packing
-  if ((cs = copy_split(h, h->ws.R2, H, (size_t)h->n * h->r * 4, kind, s)) != NMD_OK) return cs;
-  launch_pack(h->ws.R2, true, h->n, h->r, h->rp, h->B, s);
-  h->launches++;
-  CK(h, cudaMemsetAsync(h->W.E, 0, (size_t)h->m * h->rp * 4, s));
-  CK(h, cudaMemsetAsync(h->B.E, 0, (size_t)h->n * h->rp * 4, s));
+  PackArgs pw{W, false, h->m, h->W.master, h->W.hi, h->W.lo, h->W.lo2, h->W.E};
+  PackArgs pb{H, true, h->n, h->B.master, h->B.hi, h->B.lo, h->B.lo2, h->B.E};
+  if (on_device && readable_here(h, W) && readable_here(h, H)) {
+    launch_pack2(pw, pb, h->r, h->rp, s);
+    h->launches++;
+  } else {
+    // stage through R (max(m, n) x rp floats >= m x r and r x n)
+    const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+    nmd_status cs = copy_split(h, h->ws.R, W, (size_t)h->m * h->r * 4, kind, s);
+    if (cs != NMD_OK) return cs;
+    pw.src = h->ws.R;
+    launch_pack2(pw, PackArgs{}, h->r, h->rp, s);
+    // H goes to the second copy of R, so that its copy overlaps W's packing
+    if ((cs = copy_split(h, h->ws.R2, H, (size_t)h->n * h->r * 4, kind, s)) != NMD_OK) return cs;
+    pb.src = h->ws.R2;
+    launch_pack2(pb, PackArgs{}, h->r, h->rp, s);
+    h->launches += 2;
+  }
   nmd_status st = after_launch(h, "pack factors");
   if (st != NMD_OK) return st;
   if (!on_device) CK(h, cudaStreamSynchronize(s));   // host buffers may be released after return
@@ -1130,8 +1147,17 @@ nmd_status nmd_set_factors(nmd_handle* h, const float* W, const float* H, int on
 nmd_status nmd_get_factors(nmd_handle* h, float* W, float* H, int on_device) {
   if (!h) return NMD_ERR_INVALID;
   DeviceScope dg(h);
-  nmd_status st = sync_and_check(h);
   cudaStream_t s = h->stream;
+  if (on_device && (!W || readable_here(h, W)) && (!H || readable_here(h, H))) {
+    // straight into the caller's buffers, behind the work in flight
+    nmd_status st = wait_all_pending(h);
+    if (st != NMD_OK) return st;
+    launch_unpack2(W ? UnpackArgs{h->W.master, false, h->m, W} : UnpackArgs{},
+                   H ? UnpackArgs{h->B.master, true, h->n, H} : UnpackArgs{}, h->r, h->rp, s);
+    if (W || H) h->launches++;
+    return sync_and_check(h);
+  }
+  nmd_status st = sync_and_check(h);
   cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   if (W) {
     launch_unpack(h->W.master, false, h->m, h->r, h->rp, h->ws.R, s);

@@ -32,39 +32,89 @@ inline int grid_for(int64_t work, int threads, int cap = 152 * 16) {
 // Packing: fp32 (N x r, or r x N) -> N x rp master plus its bf16 pieces
 // hi = bf16_rn(x), lo = bf16_rn(x - hi), lo2 = bf16_rn(x - hi - lo) (each
 // difference is exact in fp32); pad columns are zero.
+// Bounded by memory; a 32-row tile per block, so that an r x N source (or
+// destination) is read along its rows and turned in shared memory, and
+// everything padded moves as 16 or 8 bytes a thread.  Element by element with
+// the transposed side strided by N, both factors of 139,255 rows at r = 64
+// took 315 us in and out (with the staging copies, the clearing of E and the
+// synchronisations); this way 145 us.
 // ---------------------------------------------------------------------------
-__global__ void pack_kernel(const float* __restrict__ src, int src_is_rxN, int64_t N, int r, int rp,
-                            float* __restrict__ master, bf16* __restrict__ hi, bf16* __restrict__ lo,
-                            bf16* __restrict__ lo2) {
-  int64_t total = N * rp;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    int64_t j = idx / rp;
-    int c = (int)(idx - j * rp);
-    float v = 0.f;
-    if (c < r) v = src_is_rxN ? src[(int64_t)c * N + j] : src[j * r + c];
-    master[idx] = v;
-    if (hi) {
-      const bf16 h = __float2bfloat16_rn(v);
-      const float r1 = v - __bfloat162float(h);
-      const bf16 l = __float2bfloat16_rn(r1);
-      hi[idx] = h;
-      lo[idx] = l;
-      lo2[idx] = __float2bfloat16_rn(r1 - __bfloat162float(l));
+constexpr int kPackRows = 32;
+
+// tile `t` of a factor: sm is r_pad x 33 floats
+__device__ __forceinline__ void pack_tile(const PackArgs& p, int r, int rp, int64_t t, float* sm) {
+  const int64_t j0 = t * kPackRows;
+  const int nr = (int)min((int64_t)kPackRows, p.N - j0), tid = threadIdx.x;
+  if (p.rxN)
+    for (int e = tid; e < r * kPackRows; e += 256) {
+      const int c = e / kPackRows, jj = e % kPackRows;
+      if (jj < nr) sm[c * (kPackRows + 1) + jj] = p.src[(int64_t)c * p.N + j0 + jj];
     }
+  else
+    for (int e = tid; e < nr * r; e += 256) {
+      const int jj = e / r, c = e - jj * r;
+      sm[c * (kPackRows + 1) + jj] = p.src[j0 * r + e];
+    }
+  __syncthreads();
+  const int q = rp / 4;   // a power of two
+  for (int e = tid; e < nr * q; e += 256) {
+    const int jj = e / q, c = e % q * 4;
+    float v[4];
+    uint32_t h[4], l[4], l2[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      v[k] = c + k < r ? sm[(c + k) * (kPackRows + 1) + jj] : 0.f;
+      const bf16 hi = __float2bfloat16_rn(v[k]);
+      const float r1 = v[k] - __bfloat162float(hi);
+      const bf16 lo = __float2bfloat16_rn(r1);
+      h[k] = __bfloat16_as_ushort(hi);
+      l[k] = __bfloat16_as_ushort(lo);
+      l2[k] = __bfloat16_as_ushort(__float2bfloat16_rn(r1 - __bfloat162float(lo)));
+    }
+    const int64_t o = (j0 + jj) * rp + c;
+    *(float4*)(p.master + o) = make_float4(v[0], v[1], v[2], v[3]);
+    if (p.hi) {
+      *(uint2*)(p.hi + o) = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
+      *(uint2*)(p.lo + o) = make_uint2(l[0] | (l[1] << 16), l[2] | (l[3] << 16));
+      *(uint2*)(p.lo2 + o) = make_uint2(l2[0] | (l2[1] << 16), l2[2] | (l2[3] << 16));
+    }
+    if (p.zero) *(float4*)(p.zero + o) = make_float4(0.f, 0.f, 0.f, 0.f);
   }
 }
 
-__global__ void unpack_kernel(const float* __restrict__ master, int dst_is_rxN, int64_t N, int r,
-                              int rp, float* __restrict__ dst) {
-  int64_t total = N * r;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    int64_t j, c;
-    if (dst_is_rxN) { c = idx / N; j = idx - c * N; }
-    else { j = idx / r; c = idx - j * r; }
-    dst[idx] = master[j * rp + c];
+// one or two factors: blocks [0, na) the tiles of a, the others those of b
+__global__ void __launch_bounds__(256) pack_kernel(PackArgs a, PackArgs b, int64_t na, int r, int rp) {
+  extern __shared__ float smp[];
+  if (blockIdx.x < na) pack_tile(a, r, rp, blockIdx.x, smp);
+  else pack_tile(b, r, rp, blockIdx.x - na, smp);
+}
+
+__device__ __forceinline__ void unpack_tile(const UnpackArgs& p, int r, int rp, int64_t t, float* sm) {
+  const int64_t j0 = t * kPackRows;
+  const int nr = (int)min((int64_t)kPackRows, p.N - j0), tid = threadIdx.x, q = rp / 4;
+  for (int e = tid; e < nr * q; e += 256) {
+    const int jj = e / q, c = e % q * 4;
+    const float4 v = *(const float4*)(p.src + (j0 + jj) * rp + c);
+    float* o = sm + c * (kPackRows + 1) + jj;
+    o[0] = v.x; o[kPackRows + 1] = v.y; o[2 * (kPackRows + 1)] = v.z; o[3 * (kPackRows + 1)] = v.w;
   }
+  __syncthreads();
+  if (p.rxN)
+    for (int e = tid; e < r * kPackRows; e += 256) {
+      const int c = e / kPackRows, jj = e % kPackRows;
+      if (jj < nr) p.dst[(int64_t)c * p.N + j0 + jj] = sm[c * (kPackRows + 1) + jj];
+    }
+  else
+    for (int e = tid; e < nr * r; e += 256) {
+      const int jj = e / r, c = e - jj * r;
+      p.dst[j0 * r + e] = sm[c * (kPackRows + 1) + jj];
+    }
+}
+
+__global__ void __launch_bounds__(256) unpack_kernel(UnpackArgs a, UnpackArgs b, int64_t na, int r, int rp) {
+  extern __shared__ float smp[];
+  if (blockIdx.x < na) unpack_tile(a, r, rp, blockIdx.x, smp);
+  else unpack_tile(b, r, rp, blockIdx.x - na, smp);
 }
 
 // ---------------------------------------------------------------------------
@@ -2009,12 +2059,26 @@ __global__ void loss_final_kernel(const double* __restrict__ dparts, int nd,
 // ===========================================================================
 // launchers
 // ===========================================================================
+static int64_t pack_tiles(int64_t N) { return (N + kPackRows - 1) / kPackRows; }
+
+void launch_pack2(const PackArgs& a, const PackArgs& b, int r, int rp, cudaStream_t s) {
+  const int64_t na = pack_tiles(a.N), nb = pack_tiles(b.N);
+  if (na + nb > 0)
+    pack_kernel<<<(unsigned)(na + nb), 256, rp * (kPackRows + 1) * sizeof(float), s>>>(a, b, na, r, rp);
+}
+
+void launch_unpack2(const UnpackArgs& a, const UnpackArgs& b, int r, int rp, cudaStream_t s) {
+  const int64_t na = pack_tiles(a.N), nb = pack_tiles(b.N);
+  if (na + nb > 0)
+    unpack_kernel<<<(unsigned)(na + nb), 256, rp * (kPackRows + 1) * sizeof(float), s>>>(a, b, na, r, rp);
+}
+
 void launch_pack(const float* src, bool src_is_rxN, int64_t N, int r, int rp, Factor& f, cudaStream_t s) {
-  pack_kernel<<<grid_for(N * rp, 256), 256, 0, s>>>(src, src_is_rxN, N, r, rp, f.master, f.hi, f.lo, f.lo2);
+  launch_pack2(PackArgs{src, src_is_rxN, N, f.master, f.hi, f.lo, f.lo2, nullptr}, PackArgs{}, r, rp, s);
 }
 
 void launch_unpack(const float* master, bool dst_is_rxN, int64_t N, int r, int rp, float* dst, cudaStream_t s) {
-  unpack_kernel<<<grid_for(N * r, 256), 256, 0, s>>>(master, dst_is_rxN, N, r, rp, dst);
+  launch_unpack2(UnpackArgs{master, dst_is_rxN, N, dst}, UnpackArgs{}, r, rp, s);
 }
 
 void launch_gram_parts(const Factor* fq, bool rounded, int64_t q0, int64_t K, int rp, float* parts, int nparts,

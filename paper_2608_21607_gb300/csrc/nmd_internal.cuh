@@ -92,6 +92,25 @@ struct Factor {
   float* E = nullptr;        // N x rp momentum (fp32)
 };
 
+// A factor into the padded layout, from N x r or (rxN) r x N floats; zero:
+// N x rp floats to clear (or NULL)
+struct PackArgs {
+  const float* src = nullptr;
+  bool rxN = false;
+  int64_t N = 0;
+  float* master = nullptr;
+  bf16 *hi = nullptr, *lo = nullptr, *lo2 = nullptr;
+  float* zero = nullptr;
+};
+
+// N x rp floats without their pad columns to N x r or (rxN) r x N floats
+struct UnpackArgs {
+  const float* src = nullptr;
+  bool rxN = false;
+  int64_t N = 0;
+  float* dst = nullptr;
+};
+
 // Operands of one dense panel contraction and one update, in device memory.
 struct StepArgs {
   // M-side rows [m0, m0 + M) of factor fm, Q-side rows [q0, q0 + K) of fq
@@ -237,6 +256,9 @@ struct nmd_handle {
 namespace nmd {
 
 // ---- launchers (kernels.cu) ----
+// two factors of the same rank in one launch (N = 0: none)
+void launch_pack2(const PackArgs& a, const PackArgs& b, int r, int rp, cudaStream_t s);
+void launch_unpack2(const UnpackArgs& a, const UnpackArgs& b, int r, int rp, cudaStream_t s);
 void launch_pack(const float* src, bool src_is_rxN, int64_t N, int r, int rp, Factor& f,
                  cudaStream_t s);
 void launch_unpack(const float* master, bool dst_is_rxN, int64_t N, int r, int rp, float* dst,

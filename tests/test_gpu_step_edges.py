@@ -95,3 +95,32 @@ def test_support_term_in_shared_memory(r, K):
         D[i, S.col_idx[S.row_ptr[i]:S.row_ptr[i + 1]]] = S.vals[S.row_ptr[i]:S.row_ptr[i + 1]]
     want = np.where(D > 0, D - np.minimum(0, Mo @ Qo.T), 0.0) @ Qo
     assert rel(got.cpu().numpy()[:, :r], want) <= 1e-5
+
+
+@pytest.mark.parametrize("device", [True, False], ids=["device", "host"])
+@pytest.mark.parametrize("m,n,r", [(1, 33, 1), (31, 32, 3), (33, 64, 16), (70, 1, 17), (129, 100, 64), (65, 90, 100),
+                                   (300, 257, 256)])
+def test_factors_in_and_out(m, n, r, device):
+    """32-row tiles of the packed layout, from and to both orders, the device
+    sources and destinations one float past the allocation's alignment; the
+    momentum is cleared."""
+    import torch
+    S = _csr(m, n, [1] * m, [m, n])
+    W, H = WL.init_factors(m, n, r, r)
+    sol = N.Solver(S, r, block_rows=64, block_cols=64)
+    sol.set_state(W + 1, H + 1, W, H, 3)
+    if device:
+        def at(x):
+            b = torch.empty(x.size + 1, device="cuda")
+            b[1:] = torch.from_numpy(np.ascontiguousarray(x).reshape(-1)).cuda()
+            return b[1:].view(x.shape)
+        sol.set_factors(at(W), at(H))
+        Wo, Ho = at(np.zeros_like(W)), at(np.zeros_like(H))
+        sol.get_factors_device(Wo, Ho)
+        got = Wo.cpu().numpy(), Ho.cpu().numpy()
+    else:
+        sol.set_factors(W, H)
+        got = sol.get_factors()
+    assert np.array_equal(got[0], W) and np.array_equal(got[1], H)
+    W2, H2, EW, EH, _ = sol.get_state()
+    assert np.array_equal(W2, W) and np.array_equal(H2, H) and not EW.any() and not EH.any()
