@@ -749,7 +749,7 @@ nmd_status run_step_roles(nmd_handle* h, const Roles& ro, int kind, bool do_upda
   h->cur_Ginv = Ginv;
   // The side stream computes G = Q^T Q of the Q-side rows and G^{-1}, the
   // second side stream the support term Rs of R, the main stream the dense
-  // term of R.  None reads what another writes, so they overlap; the update
+  // term of R (or the first and the last the other way round, below).  None reads what another writes, so they overlap; the update
   // joins them.
   // Gram partials over parts of 64 Q-side rows where there are at most
   // kGramParts of them, else over kGramParts equal parts
@@ -766,23 +766,34 @@ nmd_status run_step_roles(nmd_handle* h, const Roles& ro, int kind, bool do_upda
     launch_gram_parts(ro.fq, rounded, ro.q0, ro.K, h->rp, h->ws.gram_part, nparts, chunk, s);
     h->launches++;
   }
+  // Where the dense kernel is shorter than the Gram chain (bf16, one tile per CTA of
+  // at most eight 128-row chunks: 8-11 us against 12 us and more), the chain
+  // runs on the sweep's stream and the dense kernel beside it, so that the
+  // chain is not behind a wait on another stream at both ends (identity of
+  // 4,096 at r = 3: 363 -> 347 us a sweep; 600 x 400, exact, r = 4: 225 -> 205
+  // us).  With more chunks its blocks would keep the dense kernel from starting
+  // (2,048 x 2,048 at r = 64: 852 -> 975 us); outside sweeps the stream is the
+  // caller's, behind the side streams in priority.
+  const bool gram_main = need_gram && !gram_first && h->cur == h->hp && h->opt.precision == NMD_BF16 &&
+                         ro.K <= 1024 && ro.M <= 128 * h->num_sms;
+  cudaStream_t sg = gram_main ? s : h->side, sd = gram_main ? h->side : s;
   CK(h, cudaEventRecord(h->ev_fork, s));
   CK(h, cudaStreamWaitEvent(h->side, h->ev_fork, 0));
   CK(h, cudaStreamWaitEvent(h->side2, h->ev_fork, 0));
   if (need_gram) {
-    TimedScope ts(h, NMD_K_GRAM, h->side);
+    TimedScope ts(h, NMD_K_GRAM, sg);
     if (launch_gram_inv(ro.fq, rounded, ro.q0, ro.K, h->r, h->rp, h->ws.gram_part,
                         h->ws.gram_part + (size_t)kGramParts * h->rp * h->rp, nparts, chunk, (float)h->opt.ridge, G,
-                        Ginv, gsplit_of(h, Ginv), h->ws.counters + 8, h->ws.status, h->side)) {
+                        Ginv, gsplit_of(h, Ginv), h->ws.counters + 8, h->ws.status, sg)) {
       h->launches++;
     } else {
-      launch_gram_reduce(h->ws.gram_part, nparts, h->r, h->rp, (float)h->opt.ridge, G, h->side);
-      launch_chol_inv(G, h->r, h->rp, Ginv, gsplit_of(h, Ginv), h->ws.status, h->side);
+      launch_gram_reduce(h->ws.gram_part, nparts, h->r, h->rp, (float)h->opt.ridge, G, sg);
+      launch_chol_inv(G, h->r, h->rp, Ginv, gsplit_of(h, Ginv), h->ws.status, sg);
       h->launches += 2;
     }
     if (tc_update(h)) {   // the pieces of G^{-1} for the tensor-core update
       Factor gi = *gi_of(h, Ginv);
-      launch_pack(Ginv, false, h->rp, h->rp, h->rp, gi, h->side);
+      launch_pack(Ginv, false, h->rp, h->rp, h->rp, gi, sg);
       h->launches++;
     }
   }
@@ -796,22 +807,22 @@ nmd_status run_step_roles(nmd_handle* h, const Roles& ro, int kind, bool do_upda
     launch_span(h, a, ro, sp, Rs, h->side2);
   }
   if ((st = after_launch(h, "sparse correction")) != NMD_OK) return st;
-  CK(h, cudaEventRecord(h->ev_join, h->side));
   CK(h, cudaEventRecord(h->ev_join2, h->side2));
   // dense Z-panel contraction R = P(L) Q over every (M-side, Q-side) pair
-  if (range_on(h)) range_pass(h, ro, &a, s);
+  if (range_on(h)) range_pass(h, ro, &a, sd);
   {
-    TimedScope ts(h, NMD_K_DENSE);
+    TimedScope ts(h, NMD_K_DENSE, sd);
     if (h->opt.precision == NMD_SIMT) {
-      launch_panel_simt(a, R, s);
+      launch_panel_simt(a, R, sd);
       h->launches++;
     } else {
-      st = launch_panel_tc(a, R, h->ws.status, h->ws.counters, h->num_sms, s, &h->launches, nullptr, h->ws.rpart,
+      st = launch_panel_tc(a, R, h->ws.status, h->ws.counters, h->num_sms, sd, &h->launches, nullptr, h->ws.rpart,
                            kRpartRows);
     }
   }
   if (st != NMD_OK) return fail(h, st, "no tensor-core kernel for this rank/precision on this device");
   if ((st = after_launch(h, "dense panel")) != NMD_OK) return st;
+  CK(h, cudaEventRecord(h->ev_join, h->side));
   CK(h, cudaStreamWaitEvent(s, h->ev_join, 0));
   CK(h, cudaStreamWaitEvent(s, h->ev_join2, 0));
   if (do_update) {
