@@ -1081,18 +1081,23 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
           uint32_t va[32], vb[32];
           if (kv < BN || p.Lout != nullptr) {
             // a ragged last chunk (columns past the block contribute nothing),
-            // or L itself is wanted
+            // or L itself is wanted (tested once a group: a test per column cost
+            // 36.6 instead of 32.8 us at r_pad = 16, 139,255 rows against 1,393)
 #pragma unroll 1
             for (int g = g0; g < g0 + NG; ++g) {
               tmem_ld32(lcol + g * 32, va);
               tmem_wait_ld(va);
               const int64_t li = (int64_t)t * BM + row;
+              const int n = kv - g * 32;   // valid columns of this group
+              if (n < 32) {
 #pragma unroll
-              for (int i = 0; i < 32; ++i) {
-                if (g * 32 + i >= kv) va[i] = 0u;
-                else if (p.Lout != nullptr && li < p.M)   // (the bf16 mode's Z form holds -L)
-                  p.Lout[li * p.K + c * BN + g * 32 + i] =
-                      EPI == 0 && !SPLIT ? -__uint_as_float(va[i]) : __uint_as_float(va[i]);
+                for (int i = 0; i < 32; ++i) va[i] = i < n ? va[i] : 0u;
+              }
+              if (p.Lout != nullptr && li < p.M) {   // (the bf16 mode's Z form holds -L)
+                float* lrow = p.Lout + li * p.K + c * BN + g * 32;
+#pragma unroll
+                for (int i = 0; i < 32; ++i)
+                  if (i < n) lrow[i] = EPI == 0 && !SPLIT ? -__uint_as_float(va[i]) : __uint_as_float(va[i]);
               }
               to_p(va, g);
             }
