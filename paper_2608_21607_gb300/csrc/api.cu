@@ -1334,12 +1334,14 @@ nmd_status nmd_loss(nmd_handle* h, nmd_loss_out* out) {
   // v: [relu2, relu, sum_a, sum_b, sum_min, sum_max]: the dense sums cover
   // the entries off the support (SIMT: every entry, with the support part
   // subtracted again by the support pass)
+  // (a sum that is negative by rounding is zero; one that is not a number, or
+  // infinite, stays so)
   double zl2 = v[0] + v[2], err2 = v[0] + v[3];
   out->s_fro = h->s_fro;
-  out->obj = sqrt(zl2 > 0 ? zl2 : 0.0) / h->s_fro;
-  out->rmse = sqrt(err2 > 0 ? err2 : 0.0) / h->s_fro;
+  out->obj = sqrt(zl2 < 0 ? 0.0 : zl2) / h->s_fro;
+  out->rmse = sqrt(err2 < 0 ? 0.0 : err2) / h->s_fro;
   double den = v[1] + v[5];
-  out->wjd = den > 0 ? 1.0 - v[4] / den : 0.0;
+  out->wjd = den <= 0 ? 0.0 : 1.0 - v[4] / den;
   out->sum_relu2 = v[0];
   out->sum_relu = v[1];
   return NMD_OK;

@@ -741,7 +741,8 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
     const uint32_t lane_base = ((uint32_t)((warp & 3) * 32)) << 16;
     // (loss) the chunks' sums of a row, as an fp32 sum and its rounding errors
     // (exact but for the errors' own sum, 2^-48); fp64 adds, two a chunk and
-    // thread, cost more than the pass's tensor work.  Per tile into fp64.
+    // thread, cost more than the pass's tensor work.  Per tile into fp64, and
+    // before that where the fp32 sums would leave their range (see below).
     double s2 = 0.0, s1 = 0.0;
     float h2 = 0.f, l2 = 0.f, h1 = 0.f, l1 = 0.f;
     auto two_sum = [](float& h, float& l, float x) {
@@ -1132,8 +1133,19 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
         }
         if (LOSS) {
           if (SUMS) {
-            two_sum(h2, l2, (c2a.x + c2b.x) + (c2a.y + c2b.y));
-            two_sum(h1, l1, c1.x + c1.y);
+            const float x2 = (c2a.x + c2b.x) + (c2a.y + c2b.y), x1 = c1.x + c1.y;
+            // a chunk's sum of squares is finite while L is below about 2e18, a
+            // row's sum of such chunks need not be: into fp64 in time (an
+            // infinite chunk, too, whose error term would not be a number).  The
+            // plain sums, by Cauchy's inequality the smaller ones, go with them.
+            if (__any_sync(0xffffffffu, h2 + x2 > 1e38f)) {
+              s2 += (double)h2 + (double)l2 + (double)x2;
+              s1 += (double)h1 + (double)l1 + (double)x1;
+              h2 = l2 = h1 = l1 = 0.f;
+            } else {
+              two_sum(h2, l2, x2);
+              two_sum(h1, l1, x1);
+            }
           }
           fence_before();
           __syncwarp();
