@@ -35,10 +35,11 @@
 // The MMA warps run converged and predicate each tcgen05 operation on an
 // elected lane.
 // With two of them the bookkeeping of one (barrier tests, votes, branches: about
-// 200 cycles per chunk) runs while the other's MMAs keep the tensor core busy:
-// its queue holds next to nothing, a single issuer's bookkeeping is added to
-// every chunk (860 cycles per 128 x 128 chunk at r_pad = 64 against 512 of
-// products).
+// 200 cycles per chunk) runs while the other's MMAs keep the tensor core busy,
+// whose queue holds next to nothing.  (One warp for both was faster, 93 against
+// 100 us at r_pad = 64 and 158 against 183 us at r_pad = 128, 139,255 rows
+// against 4,096, only without the wait on b_lfree, that is, by relying on an
+// order between products into different accumulators that PTX does not give.)
 // Every mbarrier wait is bounded (2 s): on expiry the kernel records
 // NMD_ERR_TIMEOUT, the other roles stop at their next wait, in-flight MMAs
 // and copies are drained and TMEM is freed before the kernel returns.
@@ -61,9 +62,12 @@ using namespace tc;
 constexpr int kEpiThreads = 256;                 // two epilogue warpgroups
 constexpr int kProducerWarp = 8, kMma1Warp = 9, kMma2Warp = 10;
 constexpr int kThreads = 352;
-// The panel kernel's registers are capped at 112: the three of its warps on an
-// SM sub-partition then leave room (16,384 - 3 x 32 x 112 registers) for two
-// warps of 80 registers, an update block's share, and for a Gram block's.
+// The panel kernel's registers are capped, so that an update block fits beside
+// it on an SM: three of its warps on a sub-partition and two of the update's
+// (of 72 registers in the bf16 mode at r_pad = 64) within 16,384 registers.
+// 120 where that is as far as it goes (bf16, r_pad = 64: 139,255 rows, blocks of
+// 4,096, 9.04 ms a sweep, 9.10 at 112, 9.57 at 104, which spills, 10.93 at 128,
+// where the deferred update no longer runs beside it).
 constexpr int BM = 128;
 constexpr uint64_t kTimeoutNs = 2000000000ull;
 
@@ -386,7 +390,7 @@ __device__ __noinline__ void store_r_tile(uint32_t tmem_r, uint32_t b_rempty, fl
 // products of the chunks that the range-search mask clears.  Separate
 // instantiations, so that the kernel without them carries none of the checks.
 template <int RP, int EPI, bool SPLIT, int MODE, int SKIPM>
-__global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 104 : 112) : 168)
+__global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 120 : 112) : 168)
     panel_tc_kernel(const __grid_constant__ CUtensorMap tq_hi, const __grid_constant__ CUtensorMap tq_lo,
                     const __grid_constant__ CUtensorMap tq_lo2, const __grid_constant__ CUtensorMap tw,
                     const TcParams p) {
@@ -399,15 +403,6 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
   using C = Cfg<RP, SPLIT, LOSS, SKIPM != 0>;
   constexpr int BN = C::BN, NB = C::NB, NSTAGE = C::NSTAGE, NWB = C::NWB;
   constexpr bool VOTE = SKIPM == 1, RANGE = SKIPM == 2;
-  // One warp issues both products (see the MMA1 issuer) where a chunk's MMAs
-  // take longer than a warp's bookkeeping: 103 -> 93 us at r_pad = 64 and 167 ->
-  // 158 us at r_pad = 128 (bf16; 139,255 rows against 4,096), 537 -> 527 us at
-  // r_pad = 128 in the fp32-accurate mode.  At r_pad <= 32 two warps share the
-  // bookkeeping (65 against 81 us at r_pad = 16), and so they do in the
-  // fp32-accurate mode at r_pad = 64 (281 against 290 us), with one W buffer or
-  // as many stages as L buffers (r_pad = 256: MMA1 must not hold up MMA2 while
-  // it waits for them), and with a range-search mask.
-  constexpr bool ONE_MMA = !LOSS && !RANGE && NWB == 2 && NSTAGE > NB && (RP == 128 || (RP == 64 && !SPLIT));
   static_assert(SKIPM == 0 || (EPI == 1 && !LOSS), "skipping is a Delta-form option");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -598,8 +593,10 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
     }
   } else if (warp == kMma1Warp) {
     // ------------------------------------------------------------ MMA1 issuer
-    // L[lb] = W tile x chunk^T for every chunk of this CTA's tiles, in order;
-    // with ONE_MMA also R += P[lb] x chunk.
+    // L[lb] = W tile x chunk^T for every chunk of this CTA's tiles, in order.
+    // L[lb] may be overwritten once the second product has read P from it, which
+    // its commit on b_lfree says: products into different accumulators have no
+    // order of their own.
     int s1 = 0, l1 = 0, wb1 = 0;
     uint32_t ph_full = 0, ph_lfree = 1, ph_wfull = 0;
     ChunkWalk<RANGE> k1(p, (int)ntiles, (int)nchunks, kc0);
@@ -612,81 +609,27 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
       ph_wfull ^= (last && wb1 == 0) ? 1u : 0u;
       k1.next(p);
     };
-    if constexpr (ONE_MMA) {
-      // MMA1 runs NB chunks ahead of MMA2, and MMA1 of chunk c + NB goes right
-      // behind MMA2 of chunk c: one thread's MMAs execute in issue order, so
-      // the L buffer that MMA2(c) reads can be overwritten by the next MMA in
-      // the queue, without waiting for MMA2's completion.  The queue holds
-      // next to nothing, so what stands between two batches of MMAs adds to
-      // the chunk: each barrier test (about 60 cycles) starts one batch
-      // before its result is needed, and the state advances without branches.
-      int s2 = 0, l2 = 0, rb2 = 0;
-      uint32_t ph_pfull = 0, ph_rempty = 1;
-      ChunkWalk<RANGE> k2 = k1;
-      bool ok = true;
-      for (int i = 0; i < NB && k1.valid() && ok; ++i) {
-        ok = conv_wait(b_full + 8 * s1, ph_full, abort_flag, p.status, 3) &&
-             (!k1.first || conv_wait(b_wfull + 8 * wb1, ph_wfull, abort_flag, p.status, 2));
-        if (!ok) break;
-        fence_after();
-        const bool last = k1.last();
-        mma1(s1, l1, wb1);
-        commit_elect(b_lfull + 8 * l1);
-        if (last) commit_elect(b_wempty + 8 * wb1);
-        advance1(last);
+    // (a chunk's barriers are tested while the chunk before is issued)
+    bool ready = false;
+    while (k1.valid()) {
+      if (!ready && (!conv_wait(b_full + 8 * s1, ph_full, abort_flag, p.status, 3) ||
+                     !conv_wait(b_lfree + 8 * l1, ph_lfree, abort_flag, p.status, 4)))
+        break;
+      if (k1.first) {
+        if (!conv_wait(b_wfull + 8 * wb1, ph_wfull, abort_flag, p.status, 2)) break;
+        if (RANGE && p.skips != nullptr && lane == 0 && k1.nlive < k1.n)
+          atomicAdd(p.skips, (unsigned long long)(k1.n - k1.nlive));
       }
-      bool pready = false;
-      while (ok && k2.valid()) {
-        if (!pready && !conv_wait(b_pfull + 8 * l2, ph_pfull, abort_flag, p.status, 5)) break;
-        if (k2.first && !conv_wait(b_rempty + 8 * rb2, ph_rempty, abort_flag, p.status, 6)) break;
-        fence_after();
-        const bool fr = mbar_test_wait(b_full + 8 * s1, ph_full);
-        const bool last2 = k2.last();
-        if (!vanishes(l2, k2.first)) mma2(s2, l2, rb2, !k2.first);
-        commit_elect(b_empty + 8 * s2);
-        if (last2) commit_elect(b_rfull + 8 * rb2);
-        s2 = s2 == NSTAGE - 1 ? 0 : s2 + 1;
-        l2 = l2 == NB - 1 ? 0 : l2 + 1;
-        ph_pfull ^= l2 == 0 ? 1u : 0u;
-        if (C::NRB == 2) rb2 ^= last2 ? 1 : 0;
-        ph_rempty ^= (last2 && rb2 == 0) ? 1u : 0u;
-        k2.next(p);
-        const bool pr = mbar_test_wait(b_pfull + 8 * l2, ph_pfull);
-        if (k1.valid()) {
-          if (!__all_sync(0xffffffffu, fr) && !conv_wait(b_full + 8 * s1, ph_full, abort_flag, p.status, 3)) break;
-          if (k1.first && !conv_wait(b_wfull + 8 * wb1, ph_wfull, abort_flag, p.status, 2)) break;
-          fence_after();
-          const bool last1 = k1.last();
-          mma1(s1, l1, wb1);
-          commit_elect(b_lfull + 8 * l1);
-          if (last1) commit_elect(b_wempty + 8 * wb1);
-          advance1(last1);
-        }
-        pready = __all_sync(0xffffffffu, pr);
-      }
-    } else {
-      // (a chunk's barriers are tested while the chunk before is issued)
-      bool ready = false;
-      while (k1.valid()) {
-        if (!ready && (!conv_wait(b_full + 8 * s1, ph_full, abort_flag, p.status, 3) ||
-                       !conv_wait(b_lfree + 8 * l1, ph_lfree, abort_flag, p.status, 4)))
-          break;
-        if (k1.first) {
-          if (!conv_wait(b_wfull + 8 * wb1, ph_wfull, abort_flag, p.status, 2)) break;
-          if (RANGE && p.skips != nullptr && lane == 0 && k1.nlive < k1.n)
-            atomicAdd(p.skips, (unsigned long long)(k1.n - k1.nlive));
-        }
-        fence_after();
-        const bool last = k1.last();
-        const int s = s1, l = l1, wb = wb1;
-        advance1(last);
-        const bool next = mbar_test_wait(b_full + 8 * s1, ph_full) & mbar_test_wait(b_lfree + 8 * l1, ph_lfree);
-        mma1(s, l, wb);
-        commit_elect(b_lfull + 8 * l);
-        if (LOSS) commit_elect(b_empty + 8 * s);
-        if (last) commit_elect(b_wempty + 8 * wb);
-        ready = __all_sync(0xffffffffu, next);
-      }
+      fence_after();
+      const bool last = k1.last();
+      const int s = s1, l = l1, wb = wb1;
+      advance1(last);
+      const bool next = mbar_test_wait(b_full + 8 * s1, ph_full) & mbar_test_wait(b_lfree + 8 * l1, ph_lfree);
+      mma1(s, l, wb);
+      commit_elect(b_lfull + 8 * l);
+      if (LOSS) commit_elect(b_empty + 8 * s);
+      if (last) commit_elect(b_wempty + 8 * wb);
+      ready = __all_sync(0xffffffffu, next);
     }
     // wait until every MMA issued by this warp has completed
     commit_elect(b_drain);
@@ -700,7 +643,7 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
     // ------------------------------------------------------------ MMA2 issuer
     // R += P[lb] x chunk for every chunk once its P is in TMEM; frees the
     // shared-memory stage and the L buffer, and hands R over per tile.
-    if constexpr (!LOSS && !ONE_MMA) {
+    if constexpr (!LOSS) {
       int s2 = 0, l2 = 0, rb2 = 0;
       uint32_t ph_pfull = 0, ph_rempty = 1;
       ChunkWalk<RANGE> k2(p, (int)ntiles, (int)nchunks, kc0);
