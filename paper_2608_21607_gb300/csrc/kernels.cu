@@ -1469,7 +1469,7 @@ __global__ void __launch_bounds__(256, (RP <= 64 ? 3 : 1)) update_kernel(float* 
   float* Rb = TC ? sm : sm + RP * CW;
   bf16* GhT = reinterpret_cast<bf16*>(sm + TR * SR);
   bf16* GlT = GhT + RP * C::SB;
-  if (*(volatile int*)status != 0) return;
+  if (sticky_error(status)) return;
   const int cw0 = blockIdx.y * CW;
   const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
   const int64_t ntiles = (rows + TR - 1) / TR;
@@ -1759,7 +1759,7 @@ __global__ void __maxnreg__(RP == 64 ? 72 : 64) update_tc_kernel(float* __restri
   constexpr int TR = C::TR, SR = C::SR, SB = C::SB, NV = C::NV, NT = C::NT, KS = RP / 16;
   extern __shared__ __align__(16) float sm[];
   __shared__ int next_batch;
-  if (*(volatile int*)status != 0) return;
+  if (sticky_error(status)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t t0 = (n0 + TR - 1) / TR, ntiles = t0 + (n1 + TR - 1) / TR;
   // first row (relative to the step's M side) and row count of a tile
@@ -1922,7 +1922,11 @@ __global__ void __maxnreg__(RP == 64 ? 72 : 64) update_tc_kernel(float* __restri
     __syncthreads();   // this stage is refilled by the next iteration's copies
     t = t1;
     t1 = t2;
-    if (counter) t2 = (t2 & 3) != 3 ? t2 + 1 : 4 * (int64_t)next_batch;
+    if (counter) {
+      // (a block's batches ascend: anything else ends its walk)
+      const int64_t drawn4 = 4 * (int64_t)next_batch;
+      t2 = (t2 & 3) != 3 ? t2 + 1 : drawn4 > t2 ? drawn4 : ntiles;
+    }
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
 }

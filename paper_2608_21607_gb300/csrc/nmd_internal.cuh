@@ -82,6 +82,17 @@ struct PanelSet {
 // [1] = a detail (pivot column, row index), [2] = step counter at the error.
 constexpr int kStatusWords = 4;
 
+#ifdef __CUDACC__
+// Whether a sticky error is set, the same answer for every thread of the block
+// (which all call it).  Other blocks and kernels on other streams set the word
+// while this one starts: threads that tested it by themselves could disagree,
+// and the ones that stay would go on without the tiles, the shared counter or
+// the TMEM address that the others were to provide.
+__device__ __forceinline__ bool sticky_error(const int* status) {
+  return __syncthreads_or(*(const volatile int*)status != 0) != 0;
+}
+#endif
+
 // One factor's device buffers (N rows, rp = padded rank columns).
 struct Factor {
   int64_t rows = 0;

@@ -397,9 +397,10 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 1
   constexpr bool LOSS = MODE != 0;     // the first product only
   constexpr bool SUMS = MODE == 1, NEAREST = MODE == 2, UPDATE = MODE == 3;
   static_assert(!UPDATE || SPLIT, "the update pass splits R and G^{-1} into two pieces");
-  // the update is skipped under a sticky error (as the CUDA-core update is);
-  // every thread reads the same word before any barrier or TMEM exists
-  if (UPDATE && *(volatile int*)p.status != 0) return;
+  // the update is skipped under a sticky error (as the CUDA-core update is),
+  // before any mbarrier or TMEM exists
+  if constexpr (UPDATE)
+    if (sticky_error(p.status)) return;
   using C = Cfg<RP, SPLIT, LOSS, SKIPM != 0>;
   constexpr int BN = C::BN, NB = C::NB, NSTAGE = C::NSTAGE, NWB = C::NWB;
   constexpr bool VOTE = SKIPM == 1, RANGE = SKIPM == 2;
