@@ -5,9 +5,11 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <cuda.h>
+
 #include <algorithm>
-#include <string>
 #include <mutex>
+#include <string>
 #include <vector>
 
 #include "nmd_internal.cuh"
@@ -874,15 +876,41 @@ nmd_status run_step_roles(nmd_handle* h, const Roles& ro, int kind, bool do_upda
 
 namespace {
 
-// The four streams of a destroyed handle, kept for the next one on the same
-// device (at most kStreamSets sets; beyond that they are destroyed).  Streams
+// The current context and its id, which no other context of the process's
+// lifetime has (contexts of one device come and go: cudaDeviceReset, or a host
+// with contexts of its own); id 0 when it cannot be told.
+struct Context {
+  CUcontext ctx = nullptr;
+  unsigned long long id = 0;
+};
+Context current_context() {
+  static const auto entry = [](const char* name) {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      return (void*)nullptr;
+    }
+    return p;
+  };
+  static const auto get = (CUresult(CUDAAPI*)(CUcontext*))entry("cuCtxGetCurrent");
+  static const auto id = (CUresult(CUDAAPI*)(CUcontext, unsigned long long*))entry("cuCtxGetId");
+  Context c;
+  if (!get || !id || get(&c.ctx) != CUDA_SUCCESS || !c.ctx || id(c.ctx, &c.id) != CUDA_SUCCESS) c.id = 0;
+  return c;
+}
+
+// The four streams of a destroyed handle, kept for the next one in the same
+// context (at most kStreamSets sets; beyond that they are destroyed).  Streams
 // are mapped to hardware queues when they are created, and the second and later
 // sets of a process share queues: with them the deferred update waits behind
-// other streams' work (connectome at r = 64: 8.9 ms a sweep on the first set,
-// 9.2 and 11.2 ms on the ones after it).
+// other streams' work (connectome at r = 64: 9.0 ms a sweep on the first set,
+// 9.4 and 11.4 ms on the ones after it).  Handles that follow one another all
+// have the first set this way; handles that are alive together do not.
 constexpr size_t kStreamSets = 4;
 struct StreamSet {
-  int device;
+  Context context;
   cudaStream_t side, side2, hp, aux;
 };
 std::mutex stream_sets_mutex;
@@ -891,11 +919,19 @@ std::vector<StreamSet>& stream_sets() {
   return *v;
 }
 
+// false if there are none; notes the handle's context
 bool take_streams(nmd_handle* h) {
+  const Context now = current_context();
+  h->ctx_id = now.id;
+  if (now.id == 0) return false;
   std::lock_guard<std::mutex> lk(stream_sets_mutex);
   auto& v = stream_sets();
+  // sets of a context that is gone (its place taken by this one) went with it
+  v.erase(std::remove_if(v.begin(), v.end(),
+                         [&](const StreamSet& t) { return t.context.ctx == now.ctx && t.context.id != now.id; }),
+          v.end());
   for (size_t i = 0; i < v.size(); ++i)
-    if (v[i].device == h->device) {
+    if (v[i].context.id == now.id) {
       h->side = v[i].side;
       h->side2 = v[i].side2;
       h->hp = v[i].hp;
@@ -906,9 +942,11 @@ bool take_streams(nmd_handle* h) {
   return false;
 }
 
-// true if kept; only whole sets, idle
+// true if kept; only whole sets, idle, in their own context
 bool keep_streams(const nmd_handle* h) {
   if (!h->side || !h->side2 || !h->hp || !h->aux) return false;
+  const Context now = current_context();
+  if (now.id == 0 || now.id != h->ctx_id) return false;
   for (cudaStream_t s : {h->side, h->side2, h->hp, h->aux})
     if (cudaStreamQuery(s) != cudaSuccess) {
       cudaGetLastError();
@@ -917,7 +955,7 @@ bool keep_streams(const nmd_handle* h) {
   std::lock_guard<std::mutex> lk(stream_sets_mutex);
   auto& v = stream_sets();
   if (v.size() >= kStreamSets) return false;
-  v.push_back({h->device, h->side, h->side2, h->hp, h->aux});
+  v.push_back({now, h->side, h->side2, h->hp, h->aux});
   return true;
 }
 
@@ -1108,9 +1146,7 @@ nmd_status nmd_create(int64_t m, int64_t n, int32_t r, const int64_t* row_ptr,
   int least = 0, greatest = 0;
   e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
   const int side_prio = greatest < least ? greatest + 1 : greatest;
-  // the Gram chain before the support term: its three short kernels wait for
-  // SM room one after the other (planted 20,000^2, r = 32: 62 -> 37 us beside
-  // the support kernel, which takes 50 us either way)
+  // the Gram chain before the support term, which takes as long either way
   const int side2_prio = std::min(side_prio + 1, least);
   if (!take_streams(h)) {
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, side_prio);

@@ -252,6 +252,7 @@ struct nmd_handle {
   int64_t launches = 0;
   int num_sms = 0;
   int device = 0;
+  unsigned long long ctx_id = 0;   // the context its streams and events belong to (0: not known)
   int cc_major = 0, cc_minor = 0;
   std::string last_error;
   // kernel timing (nmd_profile): event pairs per launch, by kernel class
