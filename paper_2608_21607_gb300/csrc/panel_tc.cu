@@ -68,6 +68,8 @@ constexpr int kThreads = 352;
 // 120 where that is as far as it goes (bf16, r_pad = 64: 139,255 rows, blocks of
 // 4,096, 9.04 ms a sweep, 9.10 at 112, 9.57 at 104, which spills, 10.93 at 128,
 // where the deferred update no longer runs beside it).
+// The fp32-accurate kernel of r_pad = 64 has 128, without which it spills: 23.5 ms
+// a sweep of the same shape, 24.15 at 112.
 constexpr int BM = 128;
 constexpr uint64_t kTimeoutNs = 2000000000ull;
 
@@ -390,7 +392,7 @@ __device__ __noinline__ void store_r_tile(uint32_t tmem_r, uint32_t b_rempty, fl
 // products of the chunks that the range-search mask clears.  Separate
 // instantiations, so that the kernel without them carries none of the checks.
 template <int RP, int EPI, bool SPLIT, int MODE, int SKIPM>
-__global__ void __maxnreg__(MODE == 0 ? (RP <= 32 ? 128 : RP == 64 && !SPLIT ? 120 : 112) : 168)
+__global__ void __maxnreg__(MODE == 0 ? (RP <= 32 || (RP == 64 && SPLIT) ? 128 : RP == 64 ? 120 : 112) : 168)
     panel_tc_kernel(const __grid_constant__ CUtensorMap tq_hi, const __grid_constant__ CUtensorMap tq_lo,
                     const __grid_constant__ CUtensorMap tq_lo2, const __grid_constant__ CUtensorMap tw,
                     const TcParams p) {
