@@ -993,14 +993,20 @@ __global__ void __maxnreg__(MODE == 0 ? (RP <= 32 || (RP == 64 && SPLIT) ? 128 :
 #pragma unroll
             for (int i = 1; i < 32; ++i) gm = fmaxf(gm, __uint_as_float(v[i]));
             if (gm > nbest) {
-              bool found = false;
+              // the places of that value as bits.  Nearly every group of a row's
+              // first chunks comes here, which are all there is of a small set:
+              // 3,000 rows take 18 us, 46 with a selection of value and 64-bit
+              // index per column (30,000 rows of up to 16 columns: 260, 465)
+              uint32_t at = 0u, neg = 0u;
 #pragma unroll
-              for (int i = 0; i < 32; ++i) {
-                if (!found && __uint_as_float(v[i]) == gm) {
-                  found = true;
-                  nbest = __uint_as_float(v[i]);
-                  nidx = cb + i;
-                }
+              for (int i = 0; i < 32; ++i) at |= __uint_as_float(v[i]) == gm ? 1u << i : 0u;
+              const int first = __ffs(at) - 1;
+              nbest = gm;
+              nidx = cb + first;
+              if (gm == 0.f) {   // of zeros, too, the first one's sign
+#pragma unroll
+                for (int i = 0; i < 32; ++i) neg |= (v[i] >> 31) << i;
+                nbest = (neg >> first) & 1u ? -0.f : 0.f;
               }
             }
           } else if (SUMS) {
