@@ -441,8 +441,10 @@ struct TimedScope {
   nmd_handle* h;
   int cls;
   cudaStream_t st;
+  bool rest;   // goes on with the launch counted by the class's last scope
   cudaEvent_t a = nullptr, b = nullptr;
-  TimedScope(nmd_handle* h_, int c, cudaStream_t s_ = nullptr) : h(h_), cls(c), st(s_ ? s_ : h_->cur) {
+  TimedScope(nmd_handle* h_, int c, cudaStream_t s_ = nullptr, bool rest_ = false)
+      : h(h_), cls(c), st(s_ ? s_ : h_->cur), rest(rest_) {
     if (h->profiling) {
       a = pool_event(h);
       b = pool_event(h);
@@ -452,7 +454,7 @@ struct TimedScope {
   ~TimedScope() {
     if (a) {
       cudaEventRecord(b, st);
-      h->timed.push_back({cls, a, b});
+      h->timed.push_back({cls, a, b, rest});
     }
   }
 };
@@ -468,7 +470,7 @@ void collect_timing(nmd_handle* h) {
     float ms = 0.f;
     if (cudaEventElapsedTime(&ms, t.a, t.b) == cudaSuccess) {
       h->prof_ms[t.cls] += ms;
-      h->prof_launches[t.cls] += 1;
+      h->prof_launches[t.cls] += t.rest ? 0 : 1;
     }
     float t0 = 0.f, t1 = 0.f;
     if (tf && cudaEventElapsedTime(&t0, h->timed[0].a, t.a) == cudaSuccess &&
@@ -784,7 +786,7 @@ nmd_status run_step_roles(nmd_handle* h, const Roles& ro, int kind, bool do_upda
   CK(h, cudaStreamWaitEvent(h->side, h->ev_fork, 0));
   CK(h, cudaStreamWaitEvent(h->side2, h->ev_fork, 0));
   if (need_gram) {
-    TimedScope ts(h, NMD_K_GRAM, sg);
+    TimedScope ts(h, NMD_K_GRAM, sg, gram_first);
     if (launch_gram_inv(ro.fq, rounded, ro.q0, ro.K, h->r, h->rp, h->ws.gram_part,
                         h->ws.gram_part + (size_t)kGramParts * h->rp * h->rp, nparts, chunk, (float)h->opt.ridge, G,
                         Ginv, gsplit_of(h, Ginv), h->ws.counters + 8, h->ws.status, sg)) {

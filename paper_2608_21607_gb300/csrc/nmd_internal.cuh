@@ -258,7 +258,7 @@ struct nmd_handle {
   // kernel timing (nmd_profile): event pairs per launch, by kernel class
   bool profiling = false;
   std::vector<cudaEvent_t> event_pool;
-  struct Timed { int cls; cudaEvent_t a, b; };  // a, b recorded on the stream the class runs on
+  struct Timed { int cls; cudaEvent_t a, b; bool rest; };  // a, b recorded on the stream the class runs on
   std::vector<Timed> timed;
   double prof_ms[5] = {0, 0, 0, 0, 0};
   int64_t prof_launches[5] = {0, 0, 0, 0, 0};
