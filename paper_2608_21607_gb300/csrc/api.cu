@@ -754,8 +754,8 @@ nmd_status run_step_roles(nmd_handle* h, const Roles& ro, int kind, bool do_upda
   h->cur_Ginv = Ginv;
   // The side stream computes G = Q^T Q of the Q-side rows and G^{-1}, the
   // second side stream the support term Rs of R, the main stream the dense
-  // term of R (or the first and the last the other way round, below).  None reads what another writes, so they overlap; the update
-  // joins them.
+  // term of R (or the first and the last the other way round, below).  None
+  // reads what another writes, so they overlap; the update joins them.
   // Gram partials over parts of 64 Q-side rows where there are at most
   // kGramParts of them, else over kGramParts equal parts
   const bool rows64 = (ro.K + 63) / 64 <= kGramParts;
@@ -764,8 +764,12 @@ nmd_status run_step_roles(nmd_handle* h, const Roles& ro, int kind, bool do_upda
   // At r_pad >= 128 a dense CTA leaves no room on its SM for a Gram block: the
   // partials run ahead of the dense kernel on the main stream (17 us at r =
   // 256, 8,192 rows) instead of on the few SMs the dense grid leaves free,
-  // where they took longer than the dense kernel.
-  const bool gram_first = need_gram && h->rp >= 128;
+  // where they took longer than the dense kernel.  Not where the dense kernel is
+  // the long one, in the fp32-accurate mode with more tiles than SMs (ahead /
+  // beside, a sweep: 60,000 rows at r = 100 9.55 / 9.27 ms, 40,000 at r = 200 14.50
+  // / 14.13 ms; with 63 tiles, 8,000 rows at r = 100, 786 / 810 us).
+  const bool gram_first = need_gram && h->rp >= 128 &&
+                          (h->opt.precision == NMD_BF16 || ro.M <= 128 * (int64_t)h->num_sms);
   if (gram_first) {
     TimedScope ts(h, NMD_K_GRAM, s);
     launch_gram_parts(ro.fq, rounded, ro.q0, ro.K, h->rp, h->ws.gram_part, nparts, chunk, s);
@@ -779,7 +783,7 @@ nmd_status run_step_roles(nmd_handle* h, const Roles& ro, int kind, bool do_upda
   // us).  With more chunks its blocks would keep the dense kernel from starting
   // (2,048 x 2,048 at r = 64: 852 -> 975 us); outside sweeps the stream is the
   // caller's, behind the side streams in priority.
-  const bool gram_main = need_gram && !gram_first && h->cur == h->hp && h->opt.precision == NMD_BF16 &&
+  const bool gram_main = need_gram && h->rp <= 64 && h->cur == h->hp && h->opt.precision == NMD_BF16 &&
                          ro.K <= 1024 && ro.M <= 128 * h->num_sms;
   cudaStream_t sg = gram_main ? s : h->side, sd = gram_main ? h->side : s;
   CK(h, cudaEventRecord(h->ev_fork, s));
@@ -792,6 +796,10 @@ nmd_status run_step_roles(nmd_handle* h, const Roles& ro, int kind, bool do_upda
                         Ginv, gsplit_of(h, Ginv), h->ws.counters + 8, h->ws.status, sg)) {
       h->launches++;
     } else {
+      if (!gram_first) {
+        launch_gram_parts(ro.fq, rounded, ro.q0, ro.K, h->rp, h->ws.gram_part, nparts, chunk, sg);
+        h->launches++;
+      }
       launch_gram_reduce(h->ws.gram_part, nparts, h->r, h->rp, (float)h->opt.ridge, G, sg);
       launch_chol_inv(G, h->r, h->rp, Ginv, gsplit_of(h, Ginv), h->ws.status, sg);
       h->launches += 2;

@@ -40,8 +40,8 @@ def _two_per_row(n, seed):
                   (0.5 + g.random(2 * n)).astype(np.float32))
 
 
-def _solver(S, r, block, order=N.NMD_ALTERNATE):
-    return N.Solver(S, r, block_rows=block, block_cols=block, precision=N.NMD_BF16, order=order, eta=0.3, gamma=0.5)
+def _solver(S, r, block, precision=N.NMD_BF16):
+    return N.Solver(S, r, block_rows=block, block_cols=block, precision=precision, eta=0.3, gamma=0.5)
 
 
 def _same(a, b):
@@ -51,10 +51,10 @@ def _same(a, b):
 
 @pytest.mark.parametrize("r,n,block", [(64, 40000, 4096), (33, 40000, 4096), (50, 20001, 640), (64, 4000, 4000),
                                        (16, 40000, 4096), (128, 20001, 4096)])
-def test_sweeps_equal_serial_steps(r, n, block):
+def test_sweeps_equal_serial_steps(r, n, block, precision=N.NMD_BF16):
     S = _two_per_row(n, [r, n])
     W, H = WL.init_factors(n, n, r, r)
-    a, b = _solver(S, r, block), _solver(S, r, block)
+    a, b = _solver(S, r, block, precision), _solver(S, r, block, precision)
     a.set_factors(W, H)
     b.set_factors(W, H)
     orc = O.State(S, W.astype(np.float64), H.astype(np.float64), O.Options(block_rows=block, block_cols=block))
@@ -65,6 +65,13 @@ def test_sweeps_equal_serial_steps(r, n, block):
         a.sync()
         b.sync()
         _same(a, b)
+
+
+@pytest.mark.parametrize("r,n,block", [(64, 20001, 4096), (100, 4000, 2048), (100, 20001, 4096), (256, 20001, 8192)])
+def test_fp32_sweeps_equal_serial_steps(r, n, block):
+    """At r_pad >= 128 the Gram partials run ahead of the dense kernel up to one
+    tile per SM, beside it with more."""
+    test_sweeps_equal_serial_steps(r, n, block, N.NMD_FP32)
 
 
 @pytest.mark.parametrize("r,n,block", [(64, 40000, 4096), (16, 40000, 4096), (128, 20001, 4096), (256, 20001, 4096)])
