@@ -8,6 +8,8 @@ tiles from a counter, over the rows before and behind the next step's block.
 of the sweep is the next step's once, the first (no rows before it), the last
 (ragged) and the middle ones.  The arithmetic of a row does not depend on the
 launch that updates it, so the results are the serial steps' bit for bit.
+(The last cases have blocks of at most 1,024 rows and at most one tile per SM,
+where the Gram chain and the dense kernel change streams within sweeps.)
 
 Errors: one row's momentum makes its first update overflow, so that a block of
 the deferred launch reports it while others start; the sweep returns the error,
@@ -50,7 +52,8 @@ def _same(a, b):
 
 
 @pytest.mark.parametrize("r,n,block", [(64, 40000, 4096), (33, 40000, 4096), (50, 20001, 640), (64, 4000, 4000),
-                                       (16, 40000, 4096), (128, 20001, 4096)])
+                                       (16, 40000, 4096), (128, 20001, 4096), (3, 6000, 512), (64, 6000, 1000),
+                                       (64, 19456, 1024)])
 def test_sweeps_equal_serial_steps(r, n, block, precision=N.NMD_BF16):
     S = _two_per_row(n, [r, n])
     W, H = WL.init_factors(n, n, r, r)
