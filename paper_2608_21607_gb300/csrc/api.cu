@@ -886,6 +886,16 @@ nmd_status run_step_roles(nmd_handle* h, const Roles& ro, int kind, bool do_upda
 
 namespace {
 
+void* driver_entry(const char* name) {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+      q == cudaDriverEntryPointSuccess)
+    return p;
+  cudaGetLastError();
+  return nullptr;
+}
+
 // The current context and its id, which no other context of the process's
 // lifetime has (contexts of one device come and go: cudaDeviceReset, or a host
 // with contexts of its own); id 0 when it cannot be told.
@@ -894,18 +904,8 @@ struct Context {
   unsigned long long id = 0;
 };
 Context current_context() {
-  static const auto entry = [](const char* name) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess) {
-      cudaGetLastError();
-      return (void*)nullptr;
-    }
-    return p;
-  };
-  static const auto get = (CUresult(CUDAAPI*)(CUcontext*))entry("cuCtxGetCurrent");
-  static const auto id = (CUresult(CUDAAPI*)(CUcontext, unsigned long long*))entry("cuCtxGetId");
+  static const auto get = (CUresult(CUDAAPI*)(CUcontext*))driver_entry("cuCtxGetCurrent");
+  static const auto id = (CUresult(CUDAAPI*)(CUcontext, unsigned long long*))driver_entry("cuCtxGetId");
   Context c;
   if (!get || !id || get(&c.ctx) != CUDA_SUCCESS || !c.ctx || id(c.ctx, &c.id) != CUDA_SUCCESS) c.id = 0;
   return c;
@@ -1212,14 +1212,21 @@ nmd_status copy_split(nmd_handle* h, void* dst, const void* src, size_t bytes, c
 }
 
 // Whether kernels on the handle's device may access p: memory of that device
-// or managed memory; anything else is staged by copies.
+// (of this context, or of none, as memory pools' is) or managed memory;
+// anything else is staged by copies, which go between contexts and devices.
 bool readable_here(const nmd_handle* h, const void* p) {
+  static const auto attribute =
+      (CUresult(CUDAAPI*)(void*, CUpointer_attribute, CUdeviceptr))driver_entry("cuPointerGetAttribute");
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return (at.type == cudaMemoryTypeDevice && at.device == h->device) || at.type == cudaMemoryTypeManaged;
+  if (at.type == cudaMemoryTypeManaged) return true;
+  if (at.type != cudaMemoryTypeDevice || at.device != h->device || !at.devicePointer || !attribute) return false;
+  CUcontext owner = nullptr;
+  return attribute(&owner, CU_POINTER_ATTRIBUTE_CONTEXT, (CUdeviceptr)p) == CUDA_SUCCESS &&
+         (!owner || owner == current_context().ctx);
 }
 
 nmd_status nmd_set_factors(nmd_handle* h, const float* W, const float* H, int on_device) {

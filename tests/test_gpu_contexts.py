@@ -49,10 +49,17 @@ opts.block_rows = opts.block_cols = 100
 opts.precision = N.NMD_SIMT
 
 
-def fit():
+class Copy:   # a device copy in the current context
+    def __init__(self, a):
+        self.m = Mem(a.nbytes)
+        ok(D.cuMemcpyHtoD_v2(self.m.p, C.c_void_p(a.ctypes.data), C.c_size_t(a.nbytes)))
+    def data_ptr(self): return self.m.p.value
+
+
+def fit(w=None, h_=None):
     ws = Mem(N.nmd_workspace_bytes(S, 4, opts))
     h = N.nmd_create(S, 4, opts, ws, None)
-    N.nmd_set_factors(h, W, H, False)
+    N.nmd_set_factors(h, W if w is None else w, H if h_ is None else h_, w is not None)
     N.nmd_sweep(h)
     N.nmd_sync(h)
     state = N.nmd_get_state(h, 300, 200, 4)[:4]
@@ -62,14 +69,15 @@ def fit():
 
 
 want = fit()
+dW, dH = Copy(W), Copy(H)   # in the primary context
 for _ in range(3):   # a context that is gone, then one that may be at its address
     ctx = C.c_void_p()
     ok(D.cuCtxCreate_v2(C.byref(ctx), 0, 0))   # made current
     for _ in range(2):
-        for x, y in zip(fit(), want):
+        for x, y in zip(fit() + fit(dW, dH) + fit(Copy(W), Copy(H)), want * 3):
             assert np.array_equal(x, y)
     ok(D.cuCtxPopCurrent_v2(C.byref(C.c_void_p())))
-    for x, y in zip(fit(), want):   # in the primary context, the other one alive
+    for x, y in zip(fit() + fit(dW, dH), want * 2):   # in the primary context, the other one alive
         assert np.array_equal(x, y)
     ok(D.cuCtxDestroy_v2(ctx))
     for x, y in zip(fit(), want):
