@@ -767,8 +767,10 @@ nmd_status run_step_roles(nmd_handle* h, const Roles& ro, int kind, bool do_upda
   // where they took longer than the dense kernel.  Not where the dense kernel is
   // the long one, in the fp32-accurate mode with more tiles than SMs (ahead /
   // beside, a sweep: 60,000 rows at r = 100 9.55 / 9.27 ms, 40,000 at r = 200 14.50
-  // / 14.13 ms; with 63 tiles, 8,000 rows at r = 100, 786 / 810 us).
-  const bool gram_first = need_gram && h->rp >= 128 &&
+  // / 14.13 ms; with 63 tiles, 8,000 rows at r = 100, 786 / 810 us), and not with the
+  // range search, whose pass over the rows stands between them and leaves room
+  // (bf16, 40,000 rows at r = 200 4.76 / 4.20 ms, 60,000 at r = 100 5.65 / 5.25 ms).
+  const bool gram_first = need_gram && h->rp >= 128 && !range_on(h) &&
                           (h->opt.precision == NMD_BF16 || ro.M <= 128 * (int64_t)h->num_sms);
   if (gram_first) {
     TimedScope ts(h, NMD_K_GRAM, s);

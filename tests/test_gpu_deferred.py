@@ -42,8 +42,8 @@ def _two_per_row(n, seed):
                   (0.5 + g.random(2 * n)).astype(np.float32))
 
 
-def _solver(S, r, block, precision=N.NMD_BF16):
-    return N.Solver(S, r, block_rows=block, block_cols=block, precision=precision, eta=0.3, gamma=0.5)
+def _solver(S, r, block, precision=N.NMD_BF16, **kw):
+    return N.Solver(S, r, block_rows=block, block_cols=block, precision=precision, eta=0.3, gamma=0.5, **kw)
 
 
 def _same(a, b):
@@ -54,10 +54,10 @@ def _same(a, b):
 @pytest.mark.parametrize("r,n,block", [(64, 40000, 4096), (33, 40000, 4096), (50, 20001, 640), (64, 4000, 4000),
                                        (16, 40000, 4096), (128, 20001, 4096), (3, 6000, 512), (64, 6000, 1000),
                                        (64, 19456, 1024)])
-def test_sweeps_equal_serial_steps(r, n, block, precision=N.NMD_BF16):
+def test_sweeps_equal_serial_steps(r, n, block, precision=N.NMD_BF16, **kw):
     S = _two_per_row(n, [r, n])
     W, H = WL.init_factors(n, n, r, r)
-    a, b = _solver(S, r, block, precision), _solver(S, r, block, precision)
+    a, b = _solver(S, r, block, precision, **kw), _solver(S, r, block, precision, **kw)
     a.set_factors(W, H)
     b.set_factors(W, H)
     orc = O.State(S, W.astype(np.float64), H.astype(np.float64), O.Options(block_rows=block, block_cols=block))
@@ -75,6 +75,14 @@ def test_fp32_sweeps_equal_serial_steps(r, n, block):
     """At r_pad >= 128 the Gram partials run ahead of the dense kernel up to one
     tile per SM, beside it with more."""
     test_sweeps_equal_serial_steps(r, n, block, N.NMD_FP32)
+
+
+@pytest.mark.parametrize("precision", [N.NMD_BF16, N.NMD_FP32], ids=["bf16", "fp32"])
+@pytest.mark.parametrize("r,n,block", [(64, 6000, 2048), (100, 6000, 2048), (200, 20001, 4096)])
+def test_range_sweeps_equal_serial_steps(r, n, block, precision):
+    """With the range search the Gram chain runs beside its pass."""
+    test_sweeps_equal_serial_steps(r, n, block, precision, epilogue=N.NMD_EPI_DELTA,
+                                   skip_zero_chunks=N.NMD_SKIP_RANGE)
 
 
 @pytest.mark.parametrize("r,n,block", [(64, 40000, 4096), (16, 40000, 4096), (128, 20001, 4096), (256, 20001, 4096)])
