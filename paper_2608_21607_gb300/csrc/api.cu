@@ -765,13 +765,15 @@ nmd_status run_step_roles(nmd_handle* h, const Roles& ro, int kind, bool do_upda
   // partials run ahead of the dense kernel on the main stream (17 us at r =
   // 256, 8,192 rows) instead of on the few SMs the dense grid leaves free,
   // where they took longer than the dense kernel.  Not where the dense kernel is
-  // the long one, in the fp32-accurate mode with more tiles than SMs (ahead /
-  // beside, a sweep: 60,000 rows at r = 100 9.55 / 9.27 ms, 40,000 at r = 200 14.50
-  // / 14.13 ms; with 63 tiles, 8,000 rows at r = 100, 786 / 810 us), and not with the
-  // range search, whose pass over the rows stands between them and leaves room
-  // (bf16, 40,000 rows at r = 200 4.76 / 4.20 ms, 60,000 at r = 100 5.65 / 5.25 ms).
+  // the long one, in the fp32-accurate mode with more than 2^25 pairs of rows
+  // (ahead / beside: 60,000 rows, blocks of 4,096, r = 100 9.55 / 9.27 ms a sweep,
+  // 40,000 by 8,192 at r = 200 14.50 / 14.13 ms, eight combined steps of 8,192^2 at r =
+  // 256 3.49 / 3.42 ms; 8,000 rows by 2,560 786 / 810 us at r = 100, 2.44 / 2.54 ms at r
+  // = 256), and not with the range search, whose pass over the rows stands between
+  // them and leaves room (bf16, 40,000 rows at r = 200 4.76 / 4.20 ms, 60,000 at r =
+  // 100 5.65 / 5.25 ms).
   const bool gram_first = need_gram && h->rp >= 128 && !range_on(h) &&
-                          (h->opt.precision == NMD_BF16 || ro.M <= 128 * (int64_t)h->num_sms);
+                          (h->opt.precision == NMD_BF16 || ro.M * ro.K <= (int64_t)1 << 25);
   if (gram_first) {
     TimedScope ts(h, NMD_K_GRAM, s);
     launch_gram_parts(ro.fq, rounded, ro.q0, ro.K, h->rp, h->ws.gram_part, nparts, chunk, s);
