@@ -218,7 +218,8 @@ nmd_status nmd_block_order(const nmd_handle* h, int64_t sweep, int32_t side, int
 
 /* Losses of the current factors (eqs. auxCost/SLloss, RMSE, WJD): a dense
  * pass over all m x n entries of L plus a correction over the support of S,
- * reduced in a fixed order in fp64.  Synchronises the stream. */
+ * reduced in a fixed order in fp64.  Sums that overflow, or are not numbers,
+ * show as infinities and NaN.  Synchronises the stream. */
 nmd_status nmd_loss(nmd_handle* h, nmd_loss_out* out);
 
 /* Waits for the stream and returns (then clears) any sticky device error. */

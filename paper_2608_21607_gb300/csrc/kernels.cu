@@ -962,8 +962,9 @@ __device__ __forceinline__ void load16(float* f, const float* p) {
   f[0] = v.x; f[1] = v.y; f[2] = v.z; f[3] = v.w;
 }
 
-// Blocks of 128 threads (of 64 registers): beside a dense CTA and an update block
-// of r_pad = 64 an SM sub-partition has 2,048 registers left, one warp's.
+// Blocks of 128 threads of few registers (56 at r_pad = 64): one warp per SM
+// sub-partition fits in what a dense CTA and, at the other ranks, an update block
+// leave of its 16,384 registers.
 constexpr int kSparseThreads = 128;
 
 template <int RP, typename T>
@@ -1298,8 +1299,8 @@ __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& hi, uin
 // that pattern, so that the address of a lane's chunk is one exclusive or away,
 // and entry slots past the item's end read a row of zeros behind the block (dot
 // product and coefficient 0) instead of being predicated.  What bounds it is
-// instruction issue (68% of the active cycles, shared memory and L2 well
-// below), so the address arithmetic counts: planted, r = 32, 2 M entries a
+// instruction issue and latency (52% of the issue slots used, 68% before the
+// address arithmetic went; shared memory and L2 well below): planted, r = 32, 2 M entries a
 // step, 38.8 us with indices, 35.8 us with addresses.  Every index lies in
 // [q0, q0 + K): the panel lists are built at create from the CSR cut to the
 // block's columns (rows, for row steps), as for the kernels above.

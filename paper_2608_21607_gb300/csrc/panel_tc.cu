@@ -21,9 +21,9 @@
 // The loss kernel runs MMA1 only, over all of W against all of B, and sums
 // max(0, L)^2 and max(0, L) over the entries outside the support of S (the
 // dense parts of eq. SLloss / eq. RMSE / eq. WJD); the support entries are
-// summed by a separate pass.  139,255 rows on both sides at r = 64: 5.5 ms of
+// summed by a separate pass.  139,255 rows on both sides at r = 64: 5.6 ms of
 // dense pass against 1.3 ms of tensor work; the rest is the epilogue's sums
-// and, on rows of many entries, finding the support columns (3.4 ms with one
+// and, on rows of many entries, finding the support columns (3.5 ms with one
 // entry a row).
 //
 // Warp roles (352 threads, one CTA per SM, persistent over M tiles):
